@@ -123,7 +123,8 @@ typedef enum { LAMB_PHI_IDENTITY = 0, LAMB_PHI_CLIP = 1 } lamb_phi_t;
 #define LAMB_STATUS_BAD_STEP  0x2u      /* *d_step < 1 with bias correction:
                                            the step was skipped, nothing was
                                            written                          */
-#define LAMB_STATUS_WAIT_TIMEOUT 0x4u   /* on-chip: a wait for the other
+#define LAMB_STATUS_WAIT_TIMEOUT 0x4u   /* on-chip, and AUTO's one-launch
+                                           two-pass steps: a wait for other
                                            CTAs' partial sums inside the
                                            kernel (wait_limit_ms) gave up
                                            and the rest of the launch gave up
@@ -164,7 +165,16 @@ typedef struct {
                                      two-pass; on such an on-chip plan,
                                      lars_step over more than one round runs
                                      the two-pass kernels
-                                     (lamb_plan_get_info reports the choice) */
+                                     (lamb_plan_get_info reports the choice).
+                                     A two-pass plan made by AUTO runs its
+                                     steps without the gradient check as ONE
+                                     launch where most of the layout fits the
+                                     SMs in turn: a chunk's w and u stay on
+                                     the SM until its tensor's ratio is known
+                                     (28 B of HBM traffic per parameter).  m,
+                                     v and u are the two kernels' bit for bit;
+                                     the norms are summed in another fixed
+                                     order                                  */
 #define LAMB_ALGO_TWO_PASS 1      /* two streaming kernels per step: 40 B of
                                      HBM traffic per parameter (bf16 g/copy) */
 /* 2 is not assigned (plan creation rejects it)                           */
@@ -195,17 +205,17 @@ typedef struct {
   int32_t blocks_per_sm; /* resident CTAs per SM for the persistent grid;
                             0 = as many as the occupancy calculator allows */
   int32_t algorithm;     /* LAMB_ALGO_*                                     */
-  int32_t wait_limit_ms; /* on-chip: a CTA's wait for the other CTAs'
-                            partial sums gives up after this long
-                            (LAMB_STATUS_WAIT_TIMEOUT); 0 = 1000           */
-  int32_t test_unmet_wait; /* on-chip, for tests of the give-up path only:
+  int32_t wait_limit_ms; /* on-chip and one-launch steps: a CTA's wait for
+                            the other CTAs' partial sums gives up after this
+                            long (LAMB_STATUS_WAIT_TIMEOUT); 0 = 1000       */
+  int32_t test_unmet_wait; /* the same steps, for tests of the give-up path only:
                             nonzero makes every CTA wait for partial sums
                             tagged for a launch that never comes, so the
                             first wait runs out after wait_limit_ms and the
                             launch returns with LAMB_STATUS_WAIT_TIMEOUT.  0
                             for every real use                             */
-  int32_t onchip_max_ctas; /* on-chip: at most this many CTAs (one per SM);
-                            0 = the SM count                               */
+  int32_t onchip_max_ctas; /* on-chip and one-launch steps: at most this many
+                            CTAs (one per SM); 0 = the SM count             */
   int32_t onchip_rows;   /* on-chip: rows of shared memory per CTA, at most
                             what the device holds; 0 = that maximum.  Fewer
                             rows make smaller rounds                       */
@@ -303,8 +313,10 @@ LAMB_API lamb_status_t lamb_plan_bind(lamb_plan_t plan, void* const* w,
  * and whose CTAs wait for each other's partial sums: do not run on-chip
  * steps of two plans at the same time on different streams (a wait that
  * cannot be met gives up after wait_limit_ms with LAMB_STATUS_WAIT_TIMEOUT
- * and leaves the plan unusable).  Steps of one plan, like all steps, must
- * not overlap either. */
+ * and leaves the plan unusable).  AUTO's one-launch steps are cooperative
+ * launches too; steps of two such plans on different streams take turns, as
+ * the device starts a cooperative grid only as a whole.  Steps of one plan,
+ * like all steps, must not overlap. */
 LAMB_API lamb_status_t lamb_step(lamb_plan_t plan, const lamb_hyper_t* hyper,
                         int64_t* d_step, const float* d_lr,
                         cudaStream_t stream);
@@ -395,10 +407,10 @@ LAMB_API lamb_status_t lamb_plan_get_info(lamb_plan_t plan, lamb_plan_info_t* in
  * stream around every kernel it launches (up to 4096 steps are kept).
  * lamb_plan_read_timing waits for those events, returns the number of steps
  * recorded and the summed device time of each kernel in milliseconds
- * (ms_per_kernel[0..n_kernels-1]; a two-pass step launches 2 kernels, an
- * on-chip step 1, or 3 when it streams tensors through the two-pass kernels
- * first; entries past the step's kernels are 0), and clears
- * the record. */
+ * (ms_per_kernel[0..n_kernels-1]; a two-pass step launches 2 kernels, or 1 in
+ * its one-launch form, an on-chip step 1, or 3 when it streams tensors through
+ * the two-pass kernels first; entries past the step's kernels are 0), and
+ * clears the record. */
 LAMB_API lamb_status_t lamb_plan_set_timing(lamb_plan_t plan, int32_t enable);
 LAMB_API lamb_status_t lamb_plan_read_timing(lamb_plan_t plan, int32_t* n_steps,
                                     double* ms_per_kernel, int32_t n_kernels);

@@ -13,6 +13,7 @@
 #include "lamb.h"
 #include "lamb_internal.h"
 #include "lamb_onchip.h"
+#include "lamb_stash.h"
 
 using namespace lamb;
 
@@ -128,6 +129,23 @@ struct lamb_plan {
   int oc_sub_grid[4] = {0, 0, 0, 0};
   ChunkDesc* oc_chunks = nullptr;
   TensorDesc* oc_tensors = nullptr;
+
+  // the two-pass step as one launch (st_grid > 0: plain steps take it)
+  int st_grid = 0;
+  int st_slots = 0, st_wslots = 0;
+  int st_max_keep = 0;
+  int st_n_items = 0;
+  int64_t st_wait_ns = 0;
+  int st_extra = 0;
+  double st_again = 0.0;        // share of the chunks that is read again
+  int64_t st_n_chunks = 0;      // its own chunk table
+  ChunkDesc* st_chunks = nullptr;
+  TensorDesc* st_tensors = nullptr;
+  float2* st_sums = nullptr;
+  StashItem* st_items = nullptr;
+  StashRec* st_recs = nullptr;
+  uint64_t* st_words = nullptr;
+  uint32_t* st_bar = nullptr;
 
   bool timing = false;
   int timed_steps = 0;
@@ -512,6 +530,44 @@ static lamb_status_t plan_create(const int64_t* sizes, int32_t n_tensors,
     p->oc_extra = unmet_wait;
   }
 
+  // AUTO's two-pass plans run plain steps as one launch, over its own chunks
+  std::vector<StashItem> h_items;
+  std::vector<ChunkDesc> h_st_chunks;
+  std::vector<TensorDesc> h_st_tensors;
+  if (auto_algo && algo == LAMB_ALGO_TWO_PASS && sh_world == 1) {
+    rc = stash_prepare(device, p->grad_bf16, &p->st_slots, &p->st_wslots);
+    if (rc) {
+      return cuda_fail((cudaError_t)rc, "one-launch kernel set-up");
+    }
+    int ctas = p->num_sms;
+    if (oc_max_ctas > 0 && oc_max_ctas < ctas) ctas = oc_max_ctas;
+    const int keep = stash_max_keep(p->st_slots);
+    int64_t count = 0;
+    h_st_tensors.resize((size_t)n_tensors);
+    if (plan_chunks(sizes, n_tensors, kStashChunk, nullptr, 0, &count,
+                    h_st_tensors.data(), decay_mask, err, sizeof(err)))
+      return fail(LAMB_ERR_INVALID_ARG, "%s", err);
+    // below two chunks per CTA the last chunks' ratios are all the time there is
+    if (keep > 0 && count >= 2 * (int64_t)ctas) {
+      h_st_chunks.resize((size_t)count);
+      if (plan_chunks(sizes, n_tensors, kStashChunk, h_st_chunks.data(), count,
+                      &count, h_st_tensors.data(), decay_mask, err,
+                      sizeof(err)))
+        return fail(LAMB_ERR_INVALID_ARG, "%s", err);
+      plan_stash(h_st_tensors.data(), n_tensors, ctas, keep, &h_items);
+      p->st_grid = ctas;
+      p->st_max_keep = keep;
+      p->st_n_chunks = count;
+      p->st_n_items = (int)h_items.size();
+      // chunks that go through pass 1 alone and are taken again for the update
+      p->st_again = (double)(h_items.size() - (size_t)count) / (double)count;
+      p->st_wait_ns = wait_ms * 1000000;
+      p->st_extra = unmet_wait;
+    } else {
+      h_st_tensors.clear();
+    }
+  }
+
   const size_t n = (size_t)n_tensors, c = (size_t)nch;
   size_t off = 0;
   auto carve = [&](size_t bytes) {
@@ -540,6 +596,13 @@ static lamb_status_t plan_create(const int64_t* sizes, int32_t n_tensors,
   const size_t o_oc_pieces = carve(p->h_oc_pieces.size() * sizeof(OcPiece));
   const size_t o_oc_slots = carve((size_t)p->oc_n_slots * 2 * sizeof(uint64_t));
   const size_t o_oc_bar = carve(kBarWords * sizeof(uint32_t));
+  const size_t o_st_chunks = carve(h_st_chunks.size() * sizeof(ChunkDesc));
+  const size_t o_st_tensors = carve(h_st_tensors.size() * sizeof(TensorDesc));
+  const size_t o_st_slots = carve(h_st_chunks.size() * sizeof(float2));
+  const size_t o_st_items = carve(h_items.size() * sizeof(StashItem));
+  const size_t o_st_recs = carve(h_items.size() * sizeof(StashRec));
+  const size_t o_st_words = carve(p->st_grid ? n * sizeof(uint64_t) : 0);
+  const size_t o_st_bar = carve(kStashBarWords * sizeof(uint32_t));
   p->arena_bytes = off;
   e = cudaMalloc(&p->arena, p->arena_bytes);
   if (e != cudaSuccess) {
@@ -567,6 +630,13 @@ static lamb_status_t plan_create(const int64_t* sizes, int32_t n_tensors,
   p->oc_pieces = reinterpret_cast<OcPiece*>(base + o_oc_pieces);
   p->oc_slots = reinterpret_cast<uint64_t*>(base + o_oc_slots);
   p->oc_bar = reinterpret_cast<uint32_t*>(base + o_oc_bar);
+  p->st_chunks = reinterpret_cast<ChunkDesc*>(base + o_st_chunks);
+  p->st_tensors = reinterpret_cast<TensorDesc*>(base + o_st_tensors);
+  p->st_sums = reinterpret_cast<float2*>(base + o_st_slots);
+  p->st_items = reinterpret_cast<StashItem*>(base + o_st_items);
+  p->st_recs = reinterpret_cast<StashRec*>(base + o_st_recs);
+  p->st_words = reinterpret_cast<uint64_t*>(base + o_st_words);
+  p->st_bar = reinterpret_cast<uint32_t*>(base + o_st_bar);
 
   // zero everything (tickets, counters, status, results, pointer table)
   e = cudaMemset(p->arena, 0, p->arena_bytes);
@@ -587,6 +657,17 @@ static lamb_status_t plan_create(const int64_t* sizes, int32_t n_tensors,
   if (e == cudaSuccess && !h_slices.empty())
     e = cudaMemcpy(p->oc_slices, h_slices.data(),
                    h_slices.size() * sizeof(OcSlice), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess && !h_st_chunks.empty())
+    e = cudaMemcpy(p->st_chunks, h_st_chunks.data(),
+                   h_st_chunks.size() * sizeof(ChunkDesc),
+                   cudaMemcpyHostToDevice);
+  if (e == cudaSuccess && !h_st_tensors.empty())
+    e = cudaMemcpy(p->st_tensors, h_st_tensors.data(),
+                   h_st_tensors.size() * sizeof(TensorDesc),
+                   cudaMemcpyHostToDevice);
+  if (e == cudaSuccess && !h_items.empty())
+    e = cudaMemcpy(p->st_items, h_items.data(),
+                   h_items.size() * sizeof(StashItem), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) {
     // trust ratio 1 for every tensor until a step computes it; a 0-element
     // tensor keeps it (its norms are 0, and a zero norm gives ratio 1)
@@ -686,6 +767,10 @@ lamb_status_t lamb_plan_bind(lamb_plan_t plan, void* const* w,
   if (e == cudaSuccess && !oc.empty())
     e = cudaMemcpyAsync(plan->oc_pieces, oc.data(), oc.size() * sizeof(OcPiece),
                         cudaMemcpyHostToDevice, stream);
+  if (e == cudaSuccess && plan->st_grid > 0)
+    e = (cudaError_t)launch_stash_records(
+        plan->st_items, plan->st_chunks, plan->st_tensors, plan->ptrs,
+        plan->grad_bf16, plan->st_recs, plan->st_n_items, stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
   if (e != cudaSuccess) return cuda_fail(e, "pointer table upload");
   plan->bound = true;
@@ -814,6 +899,82 @@ static int launch_onchip_step(const lamb_plan* p, const StepParams& sp,
   return rc ? -rc : n;
 }
 
+// Does the one-launch form run this step?  Not with the gradient check or the
+// skip mode (their decision needs all of g), and not where too much of the
+// layout has to be read again after all: that part runs at about 0.8 of the
+// two launches' rate (one launch / two, us: 200 tensors of 1M, none again, LAMB
+// 877 / 1207, LARS 694 / 827; one of 10M, 0.4 again, 73 / 85 and 62 / 63; 40 of
+// 8M, 0.45 again, 1950 / 1914 and 1648 / 1313; one of 30M, 0.8 again, 209 / 205
+// and 176 / 143).
+static bool stash_takes(const lamb_plan* p, uint32_t flags, bool lars) {
+  return p->st_grid > 0 &&
+         !(flags & (LAMB_FLAG_GRAD_NORM | LAMB_FLAG_SKIP_NONFINITE)) &&
+         p->st_again <= (lars ? 0.2 : 0.4);
+}
+
+// The two launches of a two-pass step, or one (stash_takes).  opt: 0 LAMB, 1
+// N-LAMB, 2 NN-LAMB, 3 LARS.  Events and return value as launch_onchip_step.
+static int launch_two_pass_step(const lamb_plan* p, const StepParams& sp,
+                                int opt, cudaStream_t stream,
+                                cudaEvent_t* ev) {
+  const bool lars = opt == 3;
+  int rc = 0;
+  if (stash_takes(p, sp.flags, lars)) {
+    StashParams q;
+    q.recs = p->st_recs;
+    q.words = p->st_words;
+    q.bar = p->st_bar;
+    q.n_items = p->st_n_items;
+    q.slots = p->st_slots;
+    q.wslots = p->st_wslots;
+    q.max_keep = p->st_max_keep;
+    q.extra_tag = p->st_extra;
+    q.wait_limit_ns = p->st_wait_ns;
+    StepParams own = sp;
+    own.chunks = p->st_chunks;
+    own.tensors = p->st_tensors;
+    own.slots = p->st_sums;
+    own.n_chunks = (int32_t)p->st_n_chunks;
+    rc = launch_stash(own, q, opt, p->grad_bf16, p->copy_bf16, p->st_grid,
+                      stream);
+    if (rc != (int)cudaErrorCooperativeLaunchTooLarge) {
+      if (!rc && ev) rc = (int)cudaEventRecord(ev[1], stream);
+      return rc ? -rc : 1;
+    }
+    cudaGetLastError();   // fewer SMs are free to this process than the
+                          // device has: the two launches need no residency
+  }
+  rc = lars ? launch_lars_pass1(sp, p->grad_bf16, p->grid[2], stream)
+            : launch_lamb_pass1(sp, opt, p->grad_bf16, p->grid[0], stream);
+  if (!rc && ev) rc = (int)cudaEventRecord(ev[1], stream);
+  if (!rc)
+    rc = lars ? launch_lars_pass2(sp, p->grad_bf16, p->copy_bf16, p->grid[3],
+                                  stream)
+              : launch_lamb_pass2(sp, opt, p->grad_bf16, p->copy_bf16,
+                                  p->grid[1], stream);
+  if (!rc && ev) rc = (int)cudaEventRecord(ev[2], stream);
+  return rc ? -rc : 2;
+}
+
+// One step by the plan's kernels; records its timing events.
+static lamb_status_t launch_step(lamb_plan* p, const StepParams& sp, int opt,
+                                 cudaStream_t stream, const char* what) {
+  const bool timed = p->timing && p->timed_steps < kMaxTimedSteps;
+  cudaEvent_t* ev = timed ? &p->events[(size_t)p->timed_steps *
+                                       (kKernelsPerStep + 1)]
+                          : nullptr;
+  if (timed) {
+    const cudaError_t e = cudaEventRecord(ev[0], stream);
+    if (e != cudaSuccess) return cuda_fail(e, what);
+  }
+  const int n = onchip_takes(p, sp.flags, opt == 3)
+                    ? launch_onchip_step(p, sp, opt, stream, ev)
+                    : launch_two_pass_step(p, sp, opt, stream, ev);
+  if (n < 0) return cuda_fail((cudaError_t)-n, what);
+  if (timed) p->timed_kernels[(size_t)p->timed_steps++] = (uint8_t)n;
+  return LAMB_OK;
+}
+
 static lamb_status_t run_step(lamb_plan_t plan, const lamb_hyper_t* hyper,
                               int64_t* d_step, const float* d_lr,
                               cudaStream_t stream, bool lamb) {
@@ -837,36 +998,8 @@ static lamb_status_t run_step(lamb_plan_t plan, const lamb_hyper_t* hyper,
   if (guard.err != cudaSuccess) return cuda_fail(guard.err, "cudaSetDevice");
   StepParams sp;
   fill_params(plan, hyper, d_step, d_lr, &sp);
-
-  const bool timed = plan->timing && plan->timed_steps < kMaxTimedSteps;
-  cudaEvent_t* ev = timed ? &plan->events[(size_t)plan->timed_steps *
-                                          (kKernelsPerStep + 1)]
-                          : nullptr;
-  cudaError_t e = cudaSuccess;
-  if (timed) e = cudaEventRecord(ev[0], stream);
-  int rc = (int)e;
-  if (onchip_takes(plan, hyper->flags, !lamb)) {
-    const int n = rc ? -rc : launch_onchip_step(plan, sp, lamb ? 0 : 3, stream,
-                                                 ev);
-    if (n < 0) return cuda_fail((cudaError_t)-n, lamb ? "lamb_step" : "lars_step");
-    if (timed) plan->timed_kernels[(size_t)plan->timed_steps++] = (uint8_t)n;
-    return LAMB_OK;
-  }
-  // two-pass plans, and on-chip plans with the gradient check or the skip
-  // mode
-  if (!rc)
-    rc = lamb ? launch_lamb_pass1(sp, 0, plan->grad_bf16, plan->grid[0], stream)
-              : launch_lars_pass1(sp, plan->grad_bf16, plan->grid[2], stream);
-  if (!rc && timed) rc = (int)cudaEventRecord(ev[1], stream);
-  if (!rc)
-    rc = lamb ? launch_lamb_pass2(sp, 0, plan->grad_bf16, plan->copy_bf16,
-                                  plan->grid[1], stream)
-              : launch_lars_pass2(sp, plan->grad_bf16, plan->copy_bf16,
-                                  plan->grid[3], stream);
-  if (!rc && timed) rc = (int)cudaEventRecord(ev[2], stream);
-  if (rc) return cuda_fail((cudaError_t)rc, lamb ? "lamb_step" : "lars_step");
-  if (timed) plan->timed_kernels[(size_t)plan->timed_steps++] = 2;
-  return LAMB_OK;
+  return launch_step(plan, sp, lamb ? 0 : 3, stream,
+                     lamb ? "lamb_step" : "lars_step");
 }
 
 lamb_status_t lamb_step(lamb_plan_t plan, const lamb_hyper_t* hyper,
@@ -909,28 +1042,8 @@ lamb_status_t nlamb_step(lamb_plan_t plan, const lamb_hyper_t* hyper,
   sp.psi = momentum_decay;
   sp.log2_mu_decay = momentum_decay * std::log2(0.96);
   sp.d_mu_product = d_mu_product;
-  const int nest = nesterov_second_moment ? 2 : 1;
-  const bool timed = plan->timing && plan->timed_steps < kMaxTimedSteps;
-  cudaEvent_t* ev = timed ? &plan->events[(size_t)plan->timed_steps *
-                                          (kKernelsPerStep + 1)]
-                          : nullptr;
-  int rc = timed ? (int)cudaEventRecord(ev[0], stream) : 0;
-  if (onchip_takes(plan, hyper->flags, false)) {
-    const int n = rc ? -rc : launch_onchip_step(plan, sp, nest, stream, ev);
-    if (n < 0) return cuda_fail((cudaError_t)-n, "nlamb_step");
-    if (timed) plan->timed_kernels[(size_t)plan->timed_steps++] = (uint8_t)n;
-    return LAMB_OK;
-  }
-  if (!rc)
-    rc = launch_lamb_pass1(sp, nest, plan->grad_bf16, plan->grid[0], stream);
-  if (!rc && timed) rc = (int)cudaEventRecord(ev[1], stream);
-  if (!rc)
-    rc = launch_lamb_pass2(sp, nest, plan->grad_bf16, plan->copy_bf16,
-                           plan->grid[1], stream);
-  if (!rc && timed) rc = (int)cudaEventRecord(ev[2], stream);
-  if (rc) return cuda_fail((cudaError_t)rc, "nlamb_step");
-  if (timed) plan->timed_kernels[(size_t)plan->timed_steps++] = 2;
-  return LAMB_OK;
+  return launch_step(plan, sp, nesterov_second_moment ? 2 : 1, stream,
+                     "nlamb_step");
 }
 
 // Shared checks and parameters of the two halves of a sharded step.

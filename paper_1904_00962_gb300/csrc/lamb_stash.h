@@ -1,0 +1,107 @@
+// Tables and launcher of the one-launch form of the two-pass step
+// (lamb_stash.cu).
+//
+// HBM layout added to a plan that uses it (same arena, each piece 256-byte
+// aligned):
+//   ChunkDesc  chunks[n_chunks]     16 B  its own chunk table
+//   TensorDesc tensors[n_tensors]   32 B  and tensor table
+//   float2     slots[n_chunks]       8 B  per chunk (sum w^2, sum u^2)
+//   StashItem  items[n_items]        8 B  the work, in the order it is drawn
+//   StashRec   recs[n_items]        64 B  the same with all that a CTA needs
+//                                         to know of a chunk, made by bind
+//   uint64     words[n_tensors]      8 B  per tensor: eta rho_k, tagged with
+//                                         the launch that wrote it
+//   uint32     bar[kStashBarWords]        launch epoch, finish ticket, abort
+//                                         word, work counter
+#pragma once
+#include <stdint.h>
+
+#include <vector>
+
+#include "lamb_internal.h"
+
+namespace lamb {
+
+constexpr int kStashTile = 4 * kThreads;   // elements: one float4 per thread
+// Elements per chunk.  A chunk is kept until its tensor's last one is done, so
+// short chunks need less room (of a 4096 x 1024 tensor an SM holds 27 tiles, and
+// what it forms while the last chunk is summed); but each takes a draw and a
+// ticket.  us per step, BERT-base / BERT-large / 4,000 ragged tensors: 8,192
+// elements 510 / 1612 / 4659, 10,240 508 / 1544 / 4581, 12,288 508 / 1628 / 4667,
+// 16,384 516 / 1743 / 4869; an odd number of tiles 5-15% slower (workers take
+// them in pairs).
+constexpr int kStashChunk = 10 * kStashTile;
+constexpr int kStashRecs = 16;   // chunks a CTA has drawn and not finished
+
+// What is done with a chunk.
+enum : uint32_t {
+  kStashKeep = 0u,     // pass 1; w and u stay on the SM for the update
+  kStashPlain = 1u,    // pass 1 only (a tensor larger than the grid holds)
+  kStashReread = 2u,   // pass 2 of a kStashPlain chunk, from HBM
+  kStashEnd = 3u };    // no more work
+
+struct __align__(8) StashItem {
+  uint32_t chunk;      // chunk index, kind in the two top bits
+  int32_t keep_end;    // items up to here hold every kept chunk of the tensor
+};
+
+struct __align__(16) StashRec {
+  float* w;             // at the chunk's first element
+  const void* g;
+  float* m;
+  float* v;
+  void* copy;
+  uint32_t len_bits;    // elements (at most 2^24), kStashVec, kStashDecay, kind
+                        // in the two top bits
+  int32_t tensor;
+  int32_t chunk;
+  int32_t first, n_chunks;   // of the tensor
+  int32_t keep_end;
+};
+static_assert(sizeof(StashRec) == 64, "StashRec layout");
+constexpr uint32_t kStashVec = 1u << 28;     // float4 accesses
+constexpr uint32_t kStashDecay = 1u << 29;   // weight decay applies
+constexpr uint32_t kStashLen = (1u << 28) - 1u;
+
+// Words of the launch block (uint32 indices; each on its own 128-byte line)
+constexpr int kStashEpoch = 0;     // launches that finished
+constexpr int kStashTicket = 32;   // CTAs of the current launch that finished
+constexpr int kStashAbort = 64;    // a wait gave up: the plan is unusable
+constexpr int kStashCounter = 96;  // items drawn by the current launch
+constexpr int kStashBarWords = 128;
+
+struct StashParams {
+  const StashRec* recs;
+  uint64_t* words;
+  uint32_t* bar;
+  int32_t n_items;
+  int32_t slots;          // tiles of either half (even, odd) a CTA can keep
+  int32_t wslots;         // those of them whose w is in shared memory
+  int32_t max_keep;       // kept chunks of one tensor per CTA, at most
+  int32_t extra_tag;      // > 0 only in tests of the give-up path
+  int64_t wait_limit_ns;
+};
+
+// Kept chunks of one tensor that a CTA with room for `slots` tiles of either
+// half can always hold (planner.cpp): 0 if not even one fits.
+int32_t stash_max_keep(int32_t slots);
+// The work list of the chunk table `tensors`: every tensor's chunks in order.
+// Of a tensor with more than grid * max_keep chunks the first are kept, as many
+// as leave every CTA room for a chunk of what follows, and the rest is read
+// again, last chunk first, `grid` chunks later, when the ratio is likely there.
+void plan_stash(const TensorDesc* tensors, int32_t n, int32_t grid,
+                int32_t max_keep, std::vector<StashItem>* items);
+
+// Fills recs from the items and the plan's tables, on `stream`.
+int launch_stash_records(const StashItem* items, const ChunkDesc* chunks,
+                         const TensorDesc* tensors, const TensorPtrs* ptrs,
+                         int grad_bf16, StashRec* recs, int n_items,
+                         void* stream);
+// Launcher: opt 0 LAMB, 1 N-LAMB, 2 NN-LAMB, 3 LARS.
+int launch_stash(const StepParams& p, const StashParams& q, int opt,
+                 int grad_bf16, int copy_bf16, int grid, void* stream);
+// StashParams.slots and wslots on `device`, after the kernels' static shared
+// memory and the stages; also raises the kernels' dynamic shared-memory limit.
+int stash_prepare(int device, int grad_bf16, int* slots, int* wslots);
+
+}  // namespace lamb

@@ -16,6 +16,7 @@
 
 #include "lamb_internal.h"
 #include "lamb_onchip.h"
+#include "lamb_stash.h"
 
 namespace lamb {
 
@@ -312,6 +313,63 @@ void shard_range(const ChunkDesc* chunks, int64_t n_chunks, int32_t world,
   };
   *begin = cut(rank);
   *end = cut(rank + 1);
+}
+
+}  // namespace lamb
+
+// ---------------------------------------------------------------------------
+// Work list of the one-launch two-pass step (lamb_stash.cu).
+// ---------------------------------------------------------------------------
+namespace lamb {
+
+int32_t stash_max_keep(int32_t slots) {
+  // a full chunk's tiles fill both halves alike; the last chunk of a tensor
+  // may take one more of a half (its last len mod 4 elements).  A CTA has
+  // kStashRecs records, two of them for chunks in work.
+  static_assert(kStashChunk % (2 * kStashTile) == 0, "tiles in pairs");
+  const int32_t n = (slots - 1) / (kStashChunk / (2 * kStashTile));
+  return n < kStashRecs - 2 ? n : kStashRecs - 2;
+}
+
+void plan_stash(const TensorDesc* tensors, int32_t n, int32_t grid,
+                int32_t max_keep, std::vector<StashItem>* items) {
+  items->clear();
+  const int64_t most = (int64_t)grid * max_keep;
+  int32_t last = -1;                 // last tensor with chunks
+  for (int32_t k = 0; k < n; ++k)
+    if (tensors[k].n_chunks > 0) last = k;
+  std::vector<StashItem> again;      // to be read again, `wait` items from now
+  int64_t wait = 0;
+  auto flush = [&]() {
+    items->insert(items->end(), again.begin(), again.end());
+    again.clear();
+  };
+  for (int32_t k = 0; k < n; ++k) {
+    const int32_t first = tensors[k].first_chunk, count = tensors[k].n_chunks;
+    int64_t keep = count;
+    if (count > most)
+      keep = k == last || max_keep == 1 ? most : most - grid;
+    const size_t begin = items->size();
+    size_t end = begin;              // past the tensor's last kept chunk
+    for (int32_t j = 0; j < count; ++j) {
+      items->push_back(StashItem{(uint32_t)(first + j) |
+                                     ((j < keep ? kStashKeep : kStashPlain)
+                                      << 30), 0});
+      if (j < keep) end = items->size();
+      if (!again.empty() && --wait == 0) flush();
+    }
+    for (size_t i = begin; i < end; ++i)
+      if ((*items)[i].chunk >> 30 == kStashKeep)
+        (*items)[i].keep_end = (int32_t)end;
+    if (keep < count) {
+      flush();
+      for (int32_t j = count - 1; j >= keep; --j)
+        again.push_back(StashItem{(uint32_t)(first + j) | (kStashReread << 30),
+                                  0});
+      wait = grid;
+    }
+  }
+  flush();
 }
 
 }  // namespace lamb
