@@ -174,7 +174,9 @@ typedef struct {
                                      (28 B of HBM traffic per parameter).  m,
                                      v and u are the two kernels' bit for bit;
                                      the norms are summed in another fixed
-                                     order                                  */
+                                     order.  So does an on-chip plan made
+                                     by AUTO with several rounds and mostly
+                                     long tensors (lamb_step, nlamb_step)   */
 #define LAMB_ALGO_TWO_PASS 1      /* two streaming kernels per step: 40 B of
                                      HBM traffic per parameter (bf16 g/copy) */
 /* 2 is not assigned (plan creation rejects it)                           */

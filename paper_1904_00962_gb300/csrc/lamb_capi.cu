@@ -71,6 +71,11 @@ size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 // 4.5% slower).
 constexpr int kAutoMaxRounds = 32;
 
+// An AUTO on-chip plan's steps take the one-launch form of the two-pass step
+// from so many rounds and such a mean chunk length on.
+constexpr int kStashMinRounds = 3;
+constexpr int64_t kStashMeanChunk = 5400;
+
 struct lamb_plan {
   int device = 0;
   int n_tensors = 0;
@@ -530,11 +535,19 @@ static lamb_status_t plan_create(const int64_t* sizes, int32_t n_tensors,
     p->oc_extra = unmet_wait;
   }
 
-  // AUTO's two-pass plans run plain steps as one launch, over its own chunks
+  // AUTO's two-pass plans run plain steps as one launch, over its own chunks.
+  // So do its on-chip plans of three rounds and more, whose CTAs meet in every
+  // round, unless short tensors fill them: the launch takes each by itself (~1
+  // us of an SM), the on-chip kernel up to 16 at a time.  us per LAMB step,
+  // on-chip / one launch: ResNet-50 (7 rounds) 154 / 120, 100 ragged tensors
+  // (14) 253 / 177, 4,000 tensors of 5,500 (6) 133 / 119; 1,194 ragged ones
+  // with 5,017 elements per chunk (3) 64 / 68, 10,000 of 500 (5) 59 / 138; with
+  // two rounds 47 / 47 (6.9M parameters in 161 tensors) to 36 / 40.
   std::vector<StashItem> h_items;
   std::vector<ChunkDesc> h_st_chunks;
   std::vector<TensorDesc> h_st_tensors;
-  if (auto_algo && algo == LAMB_ALGO_TWO_PASS && sh_world == 1) {
+  if (auto_algo && sh_world == 1 &&
+      (algo == LAMB_ALGO_TWO_PASS || p->oc_n_rounds >= kStashMinRounds)) {
     rc = stash_prepare(device, p->grad_bf16, &p->st_slots, &p->st_wslots);
     if (rc) {
       return cuda_fail((cudaError_t)rc, "one-launch kernel set-up");
@@ -548,7 +561,10 @@ static lamb_status_t plan_create(const int64_t* sizes, int32_t n_tensors,
                     h_st_tensors.data(), decay_mask, err, sizeof(err)))
       return fail(LAMB_ERR_INVALID_ARG, "%s", err);
     // below two chunks per CTA the last chunks' ratios are all the time there is
-    if (keep > 0 && count >= 2 * (int64_t)ctas) {
+    const bool pays = algo == LAMB_ALGO_TWO_PASS ||
+                      (p->oc_n_rounds >= kStashMinRounds &&
+                       p->n_params >= kStashMeanChunk * count);
+    if (keep > 0 && pays && count >= 2 * (int64_t)ctas) {
       h_st_chunks.resize((size_t)count);
       if (plan_chunks(sizes, n_tensors, kStashChunk, h_st_chunks.data(), count,
                       &count, h_st_tensors.data(), decay_mask, err,
@@ -908,6 +924,7 @@ static int launch_onchip_step(const lamb_plan* p, const StepParams& sp,
 // and 176 / 143).
 static bool stash_takes(const lamb_plan* p, uint32_t flags, bool lars) {
   return p->st_grid > 0 &&
+         !(lars && p->algorithm == LAMB_ALGO_ON_CHIP) &&
          !(flags & (LAMB_FLAG_GRAD_NORM | LAMB_FLAG_SKIP_NONFINITE)) &&
          p->st_again <= (lars ? 0.2 : 0.4);
 }
@@ -967,7 +984,8 @@ static lamb_status_t launch_step(lamb_plan* p, const StepParams& sp, int opt,
     const cudaError_t e = cudaEventRecord(ev[0], stream);
     if (e != cudaSuccess) return cuda_fail(e, what);
   }
-  const int n = onchip_takes(p, sp.flags, opt == 3)
+  const int n = !stash_takes(p, sp.flags, opt == 3) &&
+                        onchip_takes(p, sp.flags, opt == 3)
                     ? launch_onchip_step(p, sp, opt, stream, ev)
                     : launch_two_pass_step(p, sp, opt, stream, ev);
   if (n < 0) return cuda_fail((cudaError_t)-n, what);

@@ -133,6 +133,42 @@ def test_one_launch_matches_the_two_pass_kernels(opt, grad, copy, misalign,
         r.plan.destroy()
 
 
+@pytest.mark.parametrize("misalign", [None, {0, 4, 6}],
+                         ids=["aligned", "unaligned"])
+def test_on_chip_plans_of_several_rounds(misalign):
+    """AUTO's on-chip plan of several rounds runs lamb_step as one launch and
+    lars_step on the two-pass kernels; one with mostly short tensors keeps the
+    on-chip kernel, whose norms are within the ratio tolerance too."""
+    sizes = [100003, 90000, 3000, 0, 65539, 5 * C + 7, 8 * C, 1025, 100001]
+    kw = dict(misalign=misalign, onchip_max_ctas=4)
+    one = Run(sizes, algorithm=B.LAMB_ALGO_AUTO, **kw)
+    two = Run(sizes, algorithm=B.LAMB_ALGO_TWO_PASS, **kw)
+    info = one.plan.info()
+    assert info["algorithm"] == B.LAMB_ALGO_ON_CHIP and info["n_rounds"] > 1
+    assert one.launches() == 1 and two.launches() == 2
+    (w1, *s1), r1 = one.out()
+    (w2, *s2), r2 = two.out()
+    assert _same(s1, s2)
+    for a, b in zip(r1, r2):
+        # fp64 ratios of fp32 chunk sums: an on-chip ratio, rounded to fp32,
+        # would not be this close to its own norms
+        np.testing.assert_allclose(a.cpu(), b.cpu(), rtol=2 * TOL_RATIO, atol=0)
+    rho, wn, un = r1
+    live = [k for k in range(1, len(sizes)) if sizes[k]]
+    np.testing.assert_allclose((rho * un / wn.clamp(max=10.))[live].cpu(), 1.0,
+                               rtol=1e-12)
+    for r in (one, two):
+        r.plan.destroy()
+    lars = Run(sizes, opt="lars", algorithm=B.LAMB_ALGO_AUTO, **kw)
+    assert lars.launches() == 2
+    lars.plan.destroy()
+    short = Run([900] * 400, algorithm=B.LAMB_ALGO_AUTO, onchip_max_ctas=4)
+    assert short.plan.info()["n_rounds"] > 1 and short.launches() == 1
+    rho, wn, un = short.out()[1]
+    assert not torch.equal(rho * un, wn)     # fp32: the on-chip kernel
+    short.plan.destroy()
+
+
 def test_a_layout_read_again_for_the_most_part_takes_the_two_launches():
     r = Run([60 * C, 5 * C], algorithm=B.LAMB_ALGO_AUTO, onchip_max_ctas=2)
     assert r.launches() == 2
