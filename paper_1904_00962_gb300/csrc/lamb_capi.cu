@@ -147,6 +147,7 @@ struct lamb_plan {
   ChunkDesc* st_chunks = nullptr;
   TensorDesc* st_tensors = nullptr;
   float2* st_sums = nullptr;
+  float2* st_gsums = nullptr;
   StashItem* st_items = nullptr;
   StashRec* st_recs = nullptr;
   uint64_t* st_words = nullptr;
@@ -615,6 +616,7 @@ static lamb_status_t plan_create(const int64_t* sizes, int32_t n_tensors,
   const size_t o_st_chunks = carve(h_st_chunks.size() * sizeof(ChunkDesc));
   const size_t o_st_tensors = carve(h_st_tensors.size() * sizeof(TensorDesc));
   const size_t o_st_slots = carve(h_st_chunks.size() * sizeof(float2));
+  const size_t o_st_gsums = carve(h_st_chunks.size() * sizeof(float2));
   const size_t o_st_items = carve(h_items.size() * sizeof(StashItem));
   const size_t o_st_recs = carve(h_items.size() * sizeof(StashRec));
   const size_t o_st_words = carve(p->st_grid ? n * sizeof(uint64_t) : 0);
@@ -649,6 +651,7 @@ static lamb_status_t plan_create(const int64_t* sizes, int32_t n_tensors,
   p->st_chunks = reinterpret_cast<ChunkDesc*>(base + o_st_chunks);
   p->st_tensors = reinterpret_cast<TensorDesc*>(base + o_st_tensors);
   p->st_sums = reinterpret_cast<float2*>(base + o_st_slots);
+  p->st_gsums = reinterpret_cast<float2*>(base + o_st_gsums);
   p->st_items = reinterpret_cast<StashItem*>(base + o_st_items);
   p->st_recs = reinterpret_cast<StashRec*>(base + o_st_recs);
   p->st_words = reinterpret_cast<uint64_t*>(base + o_st_words);
@@ -915,17 +918,16 @@ static int launch_onchip_step(const lamb_plan* p, const StepParams& sp,
   return rc ? -rc : n;
 }
 
-// Does the one-launch form run this step?  Not with the gradient check or the
-// skip mode (their decision needs all of g), and not where too much of the
-// layout has to be read again after all: that part runs at about 0.8 of the
+// Does the one-launch form run this step (after a launch that reads g alone,
+// with the gradient check or the skip mode)?  Not where too much of the layout
+// has to be read again after all: that part runs at about 0.8 of the
 // two launches' rate (one launch / two, us: 200 tensors of 1M, none again, LAMB
 // 877 / 1207, LARS 694 / 827; one of 10M, 0.4 again, 73 / 85 and 62 / 63; 40 of
 // 8M, 0.45 again, 1950 / 1914 and 1648 / 1313; one of 30M, 0.8 again, 209 / 205
 // and 176 / 143).
-static bool stash_takes(const lamb_plan* p, uint32_t flags, bool lars) {
+static bool stash_takes(const lamb_plan* p, bool lars) {
   return p->st_grid > 0 &&
          !(lars && p->algorithm == LAMB_ALGO_ON_CHIP) &&
-         !(flags & (LAMB_FLAG_GRAD_NORM | LAMB_FLAG_SKIP_NONFINITE)) &&
          p->st_again <= (lars ? 0.2 : 0.4);
 }
 
@@ -936,7 +938,7 @@ static int launch_two_pass_step(const lamb_plan* p, const StepParams& sp,
                                 cudaEvent_t* ev) {
   const bool lars = opt == 3;
   int rc = 0;
-  if (stash_takes(p, sp.flags, lars)) {
+  if (stash_takes(p, lars)) {
     StashParams q;
     q.recs = p->st_recs;
     q.words = p->st_words;
@@ -952,11 +954,20 @@ static int launch_two_pass_step(const lamb_plan* p, const StepParams& sp,
     own.tensors = p->st_tensors;
     own.slots = p->st_sums;
     own.n_chunks = (int32_t)p->st_n_chunks;
-    rc = launch_stash(own, q, opt, p->grad_bf16, p->copy_bf16, p->st_grid,
-                      stream);
+    own.grad_slots = p->st_gsums;
+    int n = 0;
+    if (sp.flags & (kFlagGradNorm | kFlagSkipNonfinite)) {
+      rc = launch_grad_check(own, opt, p->grad_bf16, p->num_sms, stream);
+      if (!rc) ++n;
+      if (!rc && ev) rc = (int)cudaEventRecord(ev[n], stream);
+    }
+    if (!rc)
+      rc = launch_stash(own, q, opt, p->grad_bf16, p->copy_bf16, p->st_grid,
+                        stream);
     if (rc != (int)cudaErrorCooperativeLaunchTooLarge) {
-      if (!rc && ev) rc = (int)cudaEventRecord(ev[1], stream);
-      return rc ? -rc : 1;
+      if (!rc) ++n;
+      if (!rc && ev) rc = (int)cudaEventRecord(ev[n], stream);
+      return rc ? -rc : n;
     }
     cudaGetLastError();   // fewer SMs are free to this process than the
                           // device has: the two launches need no residency
@@ -984,7 +995,7 @@ static lamb_status_t launch_step(lamb_plan* p, const StepParams& sp, int opt,
     const cudaError_t e = cudaEventRecord(ev[0], stream);
     if (e != cudaSuccess) return cuda_fail(e, what);
   }
-  const int n = !stash_takes(p, sp.flags, opt == 3) &&
+  const int n = !stash_takes(p, opt == 3) &&
                         onchip_takes(p, sp.flags, opt == 3)
                     ? launch_onchip_step(p, sp, opt, stream, ev)
                     : launch_two_pass_step(p, sp, opt, stream, ev);

@@ -72,28 +72,6 @@ __device__ __forceinline__ void cta_sum(float* x, float (*red)[kWarps]) {
   }
 }
 
-// The tensor that finishes last in pass 1 (gradient check only): the global
-// ||g|| as a fixed-order fp64 sum over the tensors' sum g^2, and the step's
-// decision, which pass 2 reads before it writes anything.  Warp-wide.
-__device__ __forceinline__ void finalize_grad(const StepParams& p) {
-  __threadfence();
-  const int lane = threadIdx.x & 31;
-  double a = 0.0;
-  for (int k = lane; k < p.n_tensors; k += 32) a += __ldcg(&p.gsq[k]);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
-  if (lane == 0) {
-    const uint32_t bad = atomicExch(&p.gcheck->acc, 0u);
-    p.gcheck->norm = sqrt(a);
-    p.gcheck->nonfinite = bad;
-    if (bad)
-      atomicOr(p.status, kStatusGradNonfinite |
-                             ((p.flags & kFlagSkipNonfinite) ? kStatusSkipped
-                                                             : 0u));
-    p.gcheck->done = 0u;
-  }
-}
-
 // All threads of the CTA that finished tensor k's last chunk: fixed-order
 // fp64 combine of the chunk slots -> norms and trust ratio.  Thread t adds
 // slots t, t + kThreads, ... in that order; each warp adds its lanes, then

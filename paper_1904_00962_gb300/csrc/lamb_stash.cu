@@ -129,6 +129,7 @@ struct Shared {
   uint32_t epoch, abort_word;
   uint32_t tmem;
   int abort;             // leave at once
+  int dry;               // a step that is skipped: norms only
   int issued;            // tiles whose copies have been started
   int end_seq;           // chunks this CTA drew, once known
   int end_kept;          // kept chunks among them
@@ -265,6 +266,7 @@ struct Worker {
   const int slots;         // ring slots of this half of the tiles
   const int wslots;        // those whose w is in shared memory
   const int t, half, lane;
+  const bool store;        // false: a skipped step, which forms its norms only
   const LambConsts k;
   int count = 0;                 // pairs taken
   int wslot = 0, held = 0;       // next ring slot, slots held
@@ -282,6 +284,7 @@ struct Worker {
            (threadIdx.x >> 7) * (4u * kTmemSlots)),
         slots(q.slots), wslots(q.wslots), t((int)threadIdx.x % kThreads),
         half((int)threadIdx.x / kThreads), lane((int)threadIdx.x & 31),
+        store(s.dry == 0),
         k{p.b1, p.omb1, p.b2, p.omb2, s.k.c1, s.k.c2, p.eps,
           s.k.am, s.k.ag, s.k.bv, s.k.bg} {
     htile = half;
@@ -400,8 +403,10 @@ struct Worker {
         else
           lamb_moments(g[c], m[c], v[c], k);
       }
-      st4(r.m + at, make_float4(m[0], m[1], m[2], m[3]));
-      if (kV) st4(r.v + at, make_float4(v[0], v[1], v[2], v[3]));
+      if (store) {
+        st4(r.m + at, make_float4(m[0], m[1], m[2], m[3]));
+        if (kV) st4(r.v + at, make_float4(v[0], v[1], v[2], v[3]));
+      }
     }
 #pragma unroll
     for (int c = 0; c < 4; ++c)
@@ -454,8 +459,10 @@ struct Worker {
             m = lars_momentum(g, m, w[c], r.lam, k.b1, k.omb1);
           else
             lamb_moments(g, m, v, k);
-          gm[i] = m;
-          if (kV) gv[i] = v;
+          if (store) {
+            gm[i] = m;
+            if (kV) gv[i] = v;
+          }
         }
         u[c] = direction<kOpt>(m, v, g, w[c], r.lam, k);
         aw = __fmaf_rn(w[c], w[c], aw);
@@ -615,6 +622,7 @@ __device__ __forceinline__ void draw(const StepParams& p, const StashParams& q,
     if (seq >= kStashRecs &&
         !wait_phase(sh, &sh.free[slot], phase_of(seq - kStashRecs)))
       return;
+    __syncwarp();
     // Drawn only when all that was drawn before is on its way in: work that a
     // CTA holds while its ring is full delays its tensor for every other CTA
     // (BERT-large, drawing 0 / 2 / 6 tiles early: 1503 / 1570 / 1632 us).
@@ -651,7 +659,14 @@ __device__ __forceinline__ void draw(const StepParams& p, const StashParams& q,
     __syncwarp();
     const uint32_t bits = r.len_bits;
     const int len = (int)(bits & kStashLen), k = r.tensor;
-    const uint32_t kind = bits >> 30;
+    uint32_t kind = bits >> 30;
+    if (sh.dry) {   // nothing is updated
+      if (kind == kStashReread) {
+        --seq;
+        continue;
+      }
+      kind = kStashPlain;
+    }
     const int n = chunk_tiles(len, (bits & kStashVec) != 0);
     const int ks = kseq % kStashRecs;
     if (kind == kStashKeep && kseq >= kStashRecs &&
@@ -866,6 +881,7 @@ __global__ void __launch_bounds__(kStashThreads, 1)
   if (warp == kDrawer && lane == 0) {
     sh.lr = (p.flags & kFlagLrSchedule) ? 0.f : *p.d_lr;
     sh.abort = 0;
+    sh.dry = (p.flags & kFlagSkipNonfinite) && p.gcheck->nonfinite;
     sh.issued = 0;
     sh.end_seq = sh.end_kept = 0x7fffffff;
   }
@@ -940,9 +956,141 @@ __global__ void __launch_bounds__(kStashThreads, 1)
       atom_add_acq_rel(q.bar + kStashTicket, 1u) == gridDim.x - 1u) {
     st_relaxed_u32(q.bar + kStashTicket, 0u);
     st_relaxed_u32(q.bar + kStashEpoch, sh.epoch + 1u);
-    const StepScalars sc = *p.scal;
-    if (kNest && p.d_mu_product) *p.d_mu_product = sc.mu_prod;
-    close_step(p, sc);
+    if (!sh.dry) {
+      const StepScalars sc = *p.scal;
+      if (kNest && p.d_mu_product) *p.d_mu_product = sc.mu_prod;
+      close_step(p, sc);
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Gradient check before the step: reads g alone (2 or 4 B per parameter), so
+// that the step's decision is known before anything is written and the step can
+// run as one launch: 30 B per parameter with bf16 g and copy, where the two
+// kernels' skip mode moves 42 (BERT-large: 2096 us).  One warp per chunk; a lane
+// keeps 10 loads of 16 bytes in flight and adds in 8 accumulators (40 elements
+// each): 117 us of BERT-large's 1630, 5.7 TB/s.  The tensor's last
+// warp forms ||g_k||, the last tensor's the global norm and the decision, both
+// in a fixed order.
+// ---------------------------------------------------------------------------
+constexpr int kCheckLoads = 10;
+
+// 16 or 8 bytes of gradients, widened: n of them.
+__device__ __forceinline__ void widen(const float4& x, float (&g)[4]) {
+  g[0] = x.x;
+  g[1] = x.y;
+  g[2] = x.z;
+  g[3] = x.w;
+}
+__device__ __forceinline__ void widen(const uint2& x, float (&g)[4]) {
+  g[0] = __uint_as_float(x.x << 16);
+  g[1] = __uint_as_float(x.x & 0xffff0000u);
+  g[2] = __uint_as_float(x.y << 16);
+  g[3] = __uint_as_float(x.y & 0xffff0000u);
+}
+__device__ __forceinline__ void widen(const uint4& x, float (&g)[8]) {
+  float a[4], b[4];
+  widen(make_uint2(x.x, x.y), a);
+  widen(make_uint2(x.z, x.w), b);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    g[i] = a[i];
+    g[4 + i] = b[i];
+  }
+}
+
+// Adds the squares of n loads of type V at p, kN gradients each.
+template <typename V, int kN>
+__device__ __forceinline__ void check_run(const void* p, int n, float (&a)[8],
+                                          float& z) {
+  const V* v = static_cast<const V*>(p);
+  for (int base = (int)(threadIdx.x & 31); base < n;
+       base += 32 * kCheckLoads) {
+    V x[kCheckLoads];
+#pragma unroll
+    for (int i = 0; i < kCheckLoads; ++i) {
+      x[i] = V{};
+      if (base + 32 * i < n) x[i] = __ldcs(v + base + 32 * i);
+    }
+#pragma unroll
+    for (int i = 0; i < kCheckLoads; ++i) {
+      float g[kN];
+      widen(x[i], g);
+#pragma unroll
+      for (int e = 0; e < kN; ++e) {
+        float& b = a[kN == 8 ? e : 4 * (i & 1) + e];
+        b = __fmaf_rn(g[e], g[e], b);
+        z = __fmaf_rn(g[e], 0.f, z);
+      }
+    }
+  }
+}
+// Returns how many elements it took.
+__device__ __forceinline__ int check_vec(const float* g, int len,
+                                         float (&a)[8], float& z) {
+  check_run<float4, 4>(g, len >> 2, a, z);
+  return len & ~3;
+}
+__device__ __forceinline__ int check_vec(const __nv_bfloat16* g, int len,
+                                         float (&a)[8], float& z) {
+  if ((uintptr_t)g % 16 == 0) {
+    check_run<uint4, 8>(g, len >> 3, a, z);
+    return len & ~7;
+  }
+  check_run<uint2, 4>(g, len >> 2, a, z);
+  return len & ~3;
+}
+
+template <typename GT>
+__global__ void __launch_bounds__(kThreads)
+    grad_check_kernel(const StepParams p, int needs_t) {
+  const int lane = threadIdx.x & 31;
+  // a step that is skipped for its step count checks nothing
+  if (needs_t && *p.d_step < 1) return;
+  const int n_warps = (int)gridDim.x * kWarps;
+  for (int c = (int)blockIdx.x * kWarps + (int)(threadIdx.x >> 5);
+       c < p.n_chunks; c += n_warps) {
+    const ChunkDesc ch = p.chunks[c];
+    const TensorDesc td = p.tensors[ch.tensor];
+    const TensorPtrs tp = p.ptrs[ch.tensor];
+    const GT* g = static_cast<const GT*>(tp.g) + ch.offset;
+    float a[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, z = 0.f;
+    const int from = tp.vec_ok ? check_vec(g, ch.len, a, z) : 0;
+    for (int base = from + lane; base < ch.len; base += 32 * 8) {
+      float x[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        x[i] = base + 32 * i < ch.len ? ld_grad1(g + base + 32 * i) : 0.f;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        a[i] = __fmaf_rn(x[i], x[i], a[i]);
+        z = __fmaf_rn(x[i], 0.f, z);
+      }
+    }
+    const float s = warp_sum(((a[0] + a[1]) + (a[2] + a[3])) +
+                             ((a[4] + a[5]) + (a[6] + a[7])));
+    z = warp_sum(z);
+    int last = 0;
+    if (lane == 0) {
+      p.grad_slots[c] = make_float2(s, z);
+      last = atom_add_acq_rel(&p.tickets[ch.tensor], 1u) + 1u ==
+             (uint32_t)td.n_chunks;
+      if (last) p.tickets[ch.tensor] = 0u;
+    }
+    if (!__shfl_sync(0xffffffffu, last, 0)) continue;
+    double sum, nan;
+    combine(p.grad_slots + td.first_chunk, td.n_chunks, &sum, &nan);
+    int last_tensor = 0;
+    if (lane == 0) {
+      p.gsq[ch.tensor] = sum;
+      p.gnorm[ch.tensor] = sqrt(sum);
+      if (isnan(nan)) atomicOr(&p.gcheck->acc, 1u);
+      __threadfence();
+      last_tensor =
+          atomicAdd(&p.gcheck->done, 1u) + 1u == (uint32_t)p.n_live;
+    }
+    if (__shfl_sync(0xffffffffu, last_tensor, 0)) finalize_grad(p);
   }
 }
 
@@ -1069,6 +1217,24 @@ int launch_stash_records(const StashItem* items, const ChunkDesc* chunks,
   stash_records_kernel<<<(n_items + 255) / 256, 256, 0,
                          static_cast<cudaStream_t>(stream)>>>(
       items, chunks, tensors, ptrs, grad_bf16 ? 2 : 4, recs, n_items);
+  return (int)cudaGetLastError();
+}
+
+int launch_grad_check(const StepParams& p, int opt, int grad_bf16, int num_sms,
+                      void* stream) {
+  const int needs_t =
+      opt == 1 || opt == 2 ||
+      (opt == 0 && (p.flags & kFlagBiasCorrection)) ? 1 : 0;
+  // more CTAs than are resident: a warp's chunk is short, and the scheduler
+  // evens them out (BERT-large: 5 per SM 142 us, 8 127, 16 and more 120)
+  const int64_t want = ((int64_t)p.n_chunks + kWarps - 1) / kWarps;
+  const int64_t most = (int64_t)num_sms * 16;
+  const unsigned grid = (unsigned)(want < 1 ? 1 : want < most ? want : most);
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  if (grad_bf16)
+    grad_check_kernel<__nv_bfloat16><<<grid, kThreads, 0, s>>>(p, needs_t);
+  else
+    grad_check_kernel<float><<<grid, kThreads, 0, s>>>(p, needs_t);
   return (int)cudaGetLastError();
 }
 

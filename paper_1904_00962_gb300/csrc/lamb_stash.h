@@ -6,6 +6,7 @@
 //   ChunkDesc  chunks[n_chunks]     16 B  its own chunk table
 //   TensorDesc tensors[n_tensors]   32 B  and tensor table
 //   float2     slots[n_chunks]       8 B  per chunk (sum w^2, sum u^2)
+//   float2     gsums[n_chunks]       8 B  per chunk (sum g^2, sum 0*g)
 //   StashItem  items[n_items]        8 B  the work, in the order it is drawn
 //   StashRec   recs[n_items]        64 B  the same with all that a CTA needs
 //                                         to know of a chunk, made by bind
@@ -97,6 +98,10 @@ int launch_stash_records(const StashItem* items, const ChunkDesc* chunks,
                          const TensorDesc* tensors, const TensorPtrs* ptrs,
                          int grad_bf16, StashRec* recs, int n_items,
                          void* stream);
+// The gradient check over the chunk table p.chunks, into p.grad_slots and the
+// results it leads to; read by the step launched next.  opt as below.
+int launch_grad_check(const StepParams& p, int opt, int grad_bf16, int num_sms,
+                      void* stream);
 // Launcher: opt 0 LAMB, 1 N-LAMB, 2 NN-LAMB, 3 LARS.
 int launch_stash(const StepParams& p, const StashParams& q, int opt,
                  int grad_bf16, int copy_bf16, int grid, void* stream);

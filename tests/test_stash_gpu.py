@@ -133,6 +133,61 @@ def test_one_launch_matches_the_two_pass_kernels(opt, grad, copy, misalign,
         r.plan.destroy()
 
 
+def _grad_norms(r):
+    gn, total, bad = r.plan.grad_norms()
+    torch.cuda.synchronize()
+    return gn.cpu().numpy(), float(total.item()), int(bad.item())
+
+
+@pytest.mark.parametrize("opt", ["lamb", "lars", "nnlamb"])
+@pytest.mark.parametrize("grad,copy", [("f32", None), ("bf16", "bf16")])
+@pytest.mark.parametrize("misalign", [None, {0, 5, 8, 13, 18, 21}],
+                         ids=["aligned", "unaligned"])
+@pytest.mark.parametrize("bad", [None, float("nan"), float("inf")])
+@pytest.mark.parametrize("flag", ["grad_norm", "skip_nonfinite"])
+def test_gradient_check_matches_the_two_pass_kernels(opt, grad, copy, misalign,
+                                                     bad, flag):
+    """The check reads g in its own launch; norms, decision, status word and
+    what a skipped step leaves and reports are those of the two kernels."""
+    runs = []
+    for algo in (B.LAMB_ALGO_AUTO, B.LAMB_ALGO_TWO_PASS):
+        r = Run(SIZES, opt=opt, grad=grad, copy=copy, misalign=misalign,
+                flags={flag: True, "lr_schedule": (2e-3, 10, 100)},
+                algorithm=algo, onchip_max_ctas=5)
+        if bad is not None:
+            r.st.view("g", 20)[100002] = bad
+        before = r.out()[0]
+        assert r.launches() == 2
+        after, res = r.out()
+        runs.append((before, after, res, _grad_norms(r), r.plan.query()))
+        r.plan.destroy()
+    (b1, a1, r1, n1, s1), (b2, a2, r2, n2, s2) = runs
+    assert s1 == s2 and n1[2] == n2[2] == (bad is not None)
+    skipped = bad is not None and flag == "skip_nonfinite"
+    assert bool(s1 & B.LAMB_STATUS_SKIPPED) == skipped
+    if skipped:
+        assert _same(b1, a1) and _same(b2, a2)
+    m = slice(1, 2 if opt == "lars" else 3)      # m, v
+    assert _same(a1[m], a2[m]) and _same(a1[-3:], a2[-3:])
+    # a chunk's sum is fp32 over 40 (kernel: 64) elements, then trees
+    np.testing.assert_allclose(n1[0], n2[0], rtol=2 * TOL_RATIO)
+    np.testing.assert_allclose(n1[1], n2[1], rtol=2 * TOL_RATIO)
+    for a, b in zip(r1, r2):
+        np.testing.assert_allclose(a.cpu(), b.cpu(), rtol=2 * TOL_RATIO)
+
+
+def test_gradient_check_of_a_step_with_a_bad_count_does_nothing():
+    r = Run(SIZES, flags={"skip_nonfinite": True}, onchip_max_ctas=5)
+    r.st.view("g", 20)[5] = float("nan")
+    r.scalars[0].fill_(0)
+    before = r.out()[0]
+    r.step()
+    assert _same(before, r.out()[0])
+    assert r.plan.query() == B.LAMB_STATUS_BAD_STEP
+    assert _grad_norms(r)[2] == 0
+    r.plan.destroy()
+
+
 @pytest.mark.parametrize("misalign", [None, {0, 4, 6}],
                          ids=["aligned", "unaligned"])
 def test_on_chip_plans_of_several_rounds(misalign):
