@@ -27,7 +27,8 @@
 //            warp leaves the piece); per piece, the warps' sums are added in
 //            warp order into the piece's slot, tagged with the launch.
 //   exchange the CTA loads round r + 1's tables; then, for each of its
-//            tensors, it reloads the tensor's slots (written by every CTA
+//            tensors (but those it holds alone, whose sums are complete where
+//            they are formed), it reloads the tensor's slots (written by every CTA
 //            that holds a piece of it) until all carry this launch's tag.
 //            No grid-wide barrier is needed: nothing else passes between
 //            CTAs.
@@ -62,7 +63,10 @@
 // default) sets LAMB_STATUS_WAIT_TIMEOUT and an abort word; every other
 // waiter then gives up too and the launch returns.  A launch that finds the
 // abort word set does nothing; the plan must be destroyed.  The last CTA to
-// finish also closes the step (t + 1, the scheduled eta, the N-LAMB product).
+// learn the last round's ratios also closes the step (t + 1, the scheduled eta,
+// the N-LAMB product).  A grid of one CTA (up to 4,096 elements or so) is an
+// ordinary launch: with the two round trips through L2 that it does without,
+// the tiny MLP's step takes 8.2 us instead of 10.3.
 #include "lamb_device.cuh"
 #include "lamb_onchip.h"
 #include "lamb_sync.cuh"
@@ -554,24 +558,6 @@ __device__ __forceinline__ void zero_red(OcShared& sh) {
     (&sh.red[0][0])[threadIdx.x] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
-// Per piece (one warp each): the warps' sums in warp order -> its slot,
-// tagged with this launch's tag.
-__device__ __forceinline__ void piece_sums(const OcShared& sh,
-                                           const OcTables& T,
-                                           const OcParams& q, uint32_t tag) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int j = warp; j < T.np; j += kOcWarps) {
-    const float4 x = lane < kOcWarps ? sh.red[j][lane]
-                                     : make_float4(0.f, 0.f, 0.f, 0.f);
-    const F2 a = warp_sum_ff(F2{x.x, x.y}), b = warp_sum_ff(F2{x.z, x.w});
-    if (lane == 0) {
-      uint64_t* w = q.slots + 2 * (size_t)T.piece[j].slot;
-      st_relaxed_u64(w, slot_word(a, tag));
-      st_relaxed_u64(w + 1, slot_word(b, tag));
-    }
-  }
-}
-
 __device__ __forceinline__ float phi_f(float z, const StepParams& p) {
   if (p.phi == 1) {  // clip; comparisons keep NaN as NaN
     const float gl = (float)p.gamma_l, gu = (float)p.gamma_u;
@@ -581,16 +567,69 @@ __device__ __forceinline__ float phi_f(float z, const StepParams& p) {
   return z;
 }
 
+// A tensor's complete sums -> ||w||, ||u||, rho_k (Alg. 2 last line with the
+// zero-norm rule; LARS: times kappa), eta rho_k and eta lambda_k for pass 2;
+// exports where this CTA holds the tensor's first piece.
+__device__ __forceinline__ void finish_ratio(const StepParams& p,
+                                             const OcPiece& P, float coef,
+                                             float lr, bool decoupled, F2 a,
+                                             F2 b, float* s_out,
+                                             float* dd_out) {
+  const float aw = __fadd_rn(a.hi, a.lo), au = __fadd_rn(b.hi, b.lo);
+  const float wn = __fsqrt_rn(aw), un = __fsqrt_rn(au);
+  float rho = 1.f;                                   // zero-norm rule
+  if (!(wn == 0.f || un == 0.f))
+    rho = __fdiv_rn(__fmul_rn(coef, phi_f(wn, p)), un);
+  *s_out = __fmul_rn(lr, rho);
+  *dd_out = decoupled ? __fmul_rn(lr, __fmul_rn(P.decay, p.wd)) : 0.f;
+  if (P.flags & kOcExport) {
+    p.ratio[P.tensor] = (double)rho;
+    p.wnorm[P.tensor] = (double)wn;
+    p.unorm[P.tensor] = (double)un;
+    if (!isfinite(a.hi) || !isfinite(b.hi))
+      atomicOr(p.status, kStatusNonfinite);
+  }
+}
+
+// Does this CTA hold all of the piece's tensor?  Its sums then need no slot (a
+// round trip through L2), except where a test wants the wait.
+__device__ __forceinline__ bool alone(const OcPiece& P, const OcParams& q) {
+  return P.t_nslots == 1 && q.extra_arrivals == 0;
+}
+
+// Per piece (one warp each): the warps' sums in warp order -> its slot,
+// tagged with this launch's tag, or its tensor's ratio if there is no other.
+__device__ __forceinline__ void piece_sums(const StepParams& p, OcShared& sh,
+                                           OcTables& T, const OcParams& q,
+                                           uint32_t tag, float coef, float lr,
+                                           bool decoupled) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int j = warp; j < T.np; j += kOcWarps) {
+    const float4 x = lane < kOcWarps ? sh.red[j][lane]
+                                     : make_float4(0.f, 0.f, 0.f, 0.f);
+    const F2 a = warp_sum_ff(F2{x.x, x.y}), b = warp_sum_ff(F2{x.z, x.w});
+    if (lane != 0) continue;
+    const OcPiece& P = T.piece[j];
+    const uint64_t wa = slot_word(a, tag), wb = slot_word(b, tag);
+    if (alone(P, q)) {   // the values the words hold, as if they had been read
+      finish_ratio(p, P, coef, lr, decoupled, slot_value(wa), slot_value(wb),
+                   &T.s[j], &T.dd[j]);
+    } else {
+      uint64_t* w = q.slots + 2 * (size_t)P.slot;
+      st_relaxed_u64(w, wa);
+      st_relaxed_u64(w + 1, wb);
+    }
+  }
+}
+
 // Slots a lane keeps in flight when forming a ratio: a tensor has at most
 // one slot per CTA, so 8 x 32 covers a 152-SM grid in one round trip.
 constexpr int kRatioLoads = 8;
 
 // Warp-wide, per piece: the tensor's slots in slot order (lane-strided,
 // kRatioLoads slots in flight, reloaded until every word carries this
-// launch's tag, then a fixed tree) -> ||w||, ||u||, rho_k (Alg. 2 last line
-// with the zero-norm rule; LARS: times kappa), eta rho_k and eta lambda_k
-// for pass 2; exports where this CTA holds the tensor's first piece.  Returns
-// false if the wait gave up (see the file header).
+// launch's tag, then a fixed tree) and what follows from them.  Returns false
+// if the wait gave up (see the file header).
 __device__ __forceinline__ bool piece_ratio(const StepParams& p,
                                          const OcParams& q, const OcPiece& P,
                                          float coef, float lr, bool decoupled,
@@ -647,23 +686,28 @@ __device__ __forceinline__ bool piece_ratio(const StepParams& p,
   }
   a = warp_sum_ff(a);
   b = warp_sum_ff(b);
-  if (lane == 0) {
-    const float aw = __fadd_rn(a.hi, a.lo), au = __fadd_rn(b.hi, b.lo);
-    const float wn = __fsqrt_rn(aw), un = __fsqrt_rn(au);
-    float rho = 1.f;                                   // zero-norm rule
-    if (!(wn == 0.f || un == 0.f))
-      rho = __fdiv_rn(__fmul_rn(coef, phi_f(wn, p)), un);
-    *s_out = __fmul_rn(lr, rho);
-    *dd_out = decoupled ? __fmul_rn(lr, __fmul_rn(P.decay, p.wd)) : 0.f;
-    if (P.flags & kOcExport) {
-      p.ratio[P.tensor] = (double)rho;
-      p.wnorm[P.tensor] = (double)wn;
-      p.unorm[P.tensor] = (double)un;
-      if (!isfinite(a.hi) || !isfinite(b.hi))
-        atomicOr(p.status, kStatusNonfinite);
-    }
-  }
+  if (lane == 0) finish_ratio(p, P, coef, lr, decoupled, a, b, s_out, dd_out);
   return true;
+}
+
+// The last CTA to come here advances the epoch and closes the step: every CTA
+// read t (and the N-LAMB product) before its ticket, which releases it; CTA 0
+// stored the step scalars before its own.  Called by all threads, after a
+// barrier, when the last round's ratios are known, so that the ticket's round
+// trip overlaps the last update.
+template <int kNest>
+__device__ __forceinline__ void finish_launch(const StepParams& p,
+                                              const OcParams& q,
+                                              uint32_t epoch) {
+  if (threadIdx.x != kOcThreads - 32) return;   // of the warp with fewest rows
+  if (gridDim.x > 1) {
+    if (atom_add_acq_rel(q.bar + kBarTicket, 1u) != gridDim.x - 1u) return;
+    st_relaxed_u32(q.bar + kBarTicket, 0u);
+  }
+  st_relaxed_u32(q.bar + kBarEpoch, epoch + 1u);
+  const StepScalars sc = *p.scal;
+  if (kNest && p.d_mu_product) *p.d_mu_product = sc.mu_prod;
+  close_step(p, sc);
 }
 
 // ---------------------------------------------------------------------------
@@ -729,7 +773,7 @@ __global__ void __launch_bounds__(kOcThreads, 1)
   for (int r = 0; r < q.n_rounds; ++r) {
     OcTables& T = sh.tab[r & 1];
     OcTables* next = r + 1 < q.n_rounds ? &sh.tab[(r + 1) & 1] : nullptr;
-    piece_sums(sh, T, q, write_tag(sh.epoch));
+    piece_sums(p, sh, T, q, write_tag(sh.epoch), coef, lr, decoupled);
     if (threadIdx.x == 0) sh.ok = 1;
     if (next)
       load_tables(*next, q, r + 1);   // while the other CTAs finish
@@ -737,26 +781,17 @@ __global__ void __launch_bounds__(kOcThreads, 1)
       __syncthreads();
     zero_red(sh);
     for (int j = warp; j < T.np; j += kOcWarps)
-      if (!piece_ratio(p, q, T.piece[j], coef, lr, decoupled,
+      if (!alone(T.piece[j], q) &&
+          !piece_ratio(p, q, T.piece[j], coef, lr, decoupled,
                        wait_tag(q, sh.epoch), &T.s[j], &T.dd[j]))
         sh.ok = 0;
     __syncthreads();
     if (!sh.ok) return;   // the launch gave up
+    if (!next) finish_launch<kNest>(p, q, sh.epoch);
     fused_pass<kOpt, GT, kCopy>(sh, s_rows, &T, next, k, wd, decoupled);
     __syncthreads();   // T's buffer is reloaded for round r + 2
   }
-  // The last CTA to finish advances the epoch and closes the step: every
-  // CTA read t (and the N-LAMB product) before its ticket, which releases
-  // it; CTA 0 stored the step scalars before its own.
-  __syncthreads();
-  if (threadIdx.x == 0 &&
-      atom_add_acq_rel(q.bar + kBarTicket, 1u) == gridDim.x - 1u) {
-    st_relaxed_u32(q.bar + kBarTicket, 0u);
-    st_relaxed_u32(q.bar + kBarEpoch, sh.epoch + 1u);
-    const StepScalars sc = *p.scal;
-    if (kNest && p.d_mu_product) *p.d_mu_product = sc.mu_prod;
-    close_step(p, sc);
-  }
+  if (q.n_rounds == 0) finish_launch<kNest>(p, q, sh.epoch);
 }
 
 template <int kOpt, typename GT, bool kCopy>
@@ -771,7 +806,7 @@ int launch_one(const StepParams& p, const OcParams& q, int grid, int rows,
   at[0].id = cudaLaunchAttributeCooperative;
   at[0].val.cooperative = 1;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = grid > 1 ? 1 : 0;   // one CTA waits for no other
   return (int)cudaLaunchKernelEx(&cfg, onchip_step_kernel<kOpt, GT, kCopy>, p,
                                  q);
 }
