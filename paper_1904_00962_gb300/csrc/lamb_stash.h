@@ -87,9 +87,9 @@ struct StashParams {
 // half can always hold (planner.cpp): 0 if not even one fits.
 int32_t stash_max_keep(int32_t slots);
 // The work list of the chunk table `tensors`: every tensor's chunks in order.
-// Of a tensor with more than grid * max_keep chunks the first are kept, as many
-// as leave every CTA room for a chunk of what follows, and the rest is read
-// again, last chunk first, `grid` chunks later, when the ratio is likely there.
+// Of a tensor with more than grid * max_keep chunks the first that many are kept
+// and the rest is read again, last chunk first, `grid` chunks later, when the
+// ratio is likely there.
 void plan_stash(const TensorDesc* tensors, int32_t n, int32_t grid,
                 int32_t max_keep, std::vector<StashItem>* items);
 

@@ -335,9 +335,6 @@ void plan_stash(const TensorDesc* tensors, int32_t n, int32_t grid,
                 int32_t max_keep, std::vector<StashItem>* items) {
   items->clear();
   const int64_t most = (int64_t)grid * max_keep;
-  int32_t last = -1;                 // last tensor with chunks
-  for (int32_t k = 0; k < n; ++k)
-    if (tensors[k].n_chunks > 0) last = k;
   std::vector<StashItem> again;      // to be read again, `wait` items from now
   int64_t wait = 0;
   auto flush = [&]() {
@@ -346,9 +343,7 @@ void plan_stash(const TensorDesc* tensors, int32_t n, int32_t grid,
   };
   for (int32_t k = 0; k < n; ++k) {
     const int32_t first = tensors[k].first_chunk, count = tensors[k].n_chunks;
-    int64_t keep = count;
-    if (count > most)
-      keep = k == last || max_keep == 1 ? most : most - grid;
+    const int64_t keep = count < most ? count : most;
     const size_t begin = items->size();
     size_t end = begin;              // past the tensor's last kept chunk
     for (int32_t j = 0; j < count; ++j) {
