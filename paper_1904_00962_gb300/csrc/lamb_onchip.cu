@@ -55,7 +55,10 @@
 // bit-identical to theirs; only the summation of the norms differs.
 //
 // The prologue's independent loads (the abort and epoch words, eta, round 0's
-// pieces, the step count) run in separate warps and meet at one CTA barrier.
+// pieces, the step count) run in separate warps.  The fp64 constants formed from
+// the step count (~1.5 us) are the last six warps' affair: the others load the
+// tables meanwhile and start their first rows' copies, and all meet before the
+// first row is computed.
 //
 // The tags come from a launch epoch that the last CTA of a launch advances,
 // so the step can be replayed from a CUDA graph.  The wait for a tensor's
@@ -155,11 +158,9 @@ struct OcShared {
   float4 red[kOcMaxPieces][kOcWarps];  // per piece and warp: two-float
                                        // sums of w^2 (x, y) and u^2 (z, w)
   LambConsts k;
-  int64_t t;
+  ConstParts parts;
   float lr;
-  int skip;
   int ok;
-  uint32_t unused_draw;
   uint32_t epoch;        // the plan's launch epoch when this launch started
   uint32_t abort;        // the plan's abort word when this launch started
 };
@@ -465,25 +466,43 @@ __device__ __forceinline__ void pass2_row(const OcTables& T,
 // back just before the next round's copy into it is issued, so the stores of
 // one round overlap the loads of the next.  Each warp keeps one pair of rows
 // in flight.
+// `first`: the launch's first pass.  Warps below kConstWarp issue their first
+// rows, then the CTA meets (the constants are there), then the others issue
+// theirs; false if the launch has nothing to do.
+constexpr int kConstWarp = kOcWarps - 6;
+
 template <int kOpt, typename GT, bool kCopy>
-__device__ __forceinline__ void fused_pass(OcShared& sh, float4* rows,
+__device__ __forceinline__ bool fused_pass(OcShared& sh, float4* rows,
                                            const OcTables* prev,
-                                           const OcTables* cur,
-                                           const LambConsts& k, float wd,
-                                           bool decoupled) {
+                                           const OcTables* cur, float wd,
+                                           bool decoupled, bool first) {
   const int nwp = prev ? warp_rows(prev->nr) : 0;
-  const int nwc = cur ? warp_rows(cur->nr) : 0;
+  int nwc = 0;
   int done2 = 0;   // rows of the previous round written back
   typename GradRaw<GT>::T g0, g1;
   float4 v0, v1;
   OcRow r0{0u}, r1{0u};
   PieceAcc acc{F2{0.f, 0.f}, F2{0.f, 0.f}};
   for (; done2 < min(2, nwp); ++done2) pass2_row<kCopy>(*prev, rows, done2);
-  if (nwc > 0) {
-    ring_issue<kOpt, GT>(*cur, rows, 0, nwc, g0, v0, r0);
-    ring_issue<kOpt, GT>(*cur, rows, 1, nwc, g1, v1, r1);
+#pragma unroll 1
+  for (int turn = 0; turn < 2; ++turn) {
+    const bool late = first && (int)(threadIdx.x >> 5) >= kConstWarp;
+    if (cur && late == (turn == 1)) {
+      nwc = warp_rows(cur->nr);
+      ring_issue<kOpt, GT>(*cur, rows, 0, nwc, g0, v0, r0);
+      ring_issue<kOpt, GT>(*cur, rows, 1, nwc, g1, v1, r1);
+      cp_async_commit();
+    }
+    if (!first) break;
+    if (turn == 0) {
+      __syncthreads();
+      if (sh.abort || sh.parts.skip) {
+        cp_async_wait<0>();   // no copy may outlive the CTA
+        return false;
+      }
+    }
   }
-  cp_async_commit();
+  const LambConsts k = sh.k;
   for (int i = 0; i < nwc; i += 2) {
     cp_async_wait<0>();   // rows i, i + 1 have landed
     float sw0, su0, sw1 = 0.f, su1 = 0.f;
@@ -502,6 +521,7 @@ __device__ __forceinline__ void fused_pass(OcShared& sh, float4* rows,
   }
   cp_async_wait<0>();
   for (; done2 < nwp; ++done2) pass2_row<kCopy>(*prev, rows, done2);
+  return true;
 }
 
 // ---------------------------------------------------------------------------
@@ -722,54 +742,58 @@ __global__ void __launch_bounds__(kOcThreads, 1)
   constexpr int kNest = kLars ? 0 : kOpt;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
-  // ---- prologue: the launch's independent loads run in separate warps and
-  // meet at the first CTA barrier -- the abort and epoch words (the last
-  // warp), eta (the warp before it), round 0's pieces (warp 8), and the step
-  // count with the constants formed from it (warps 0-5)
-  if (warp == kOcWarps - 1 && lane == 0) {
-    sh.abort = ld_acquire_u32(q.bar + kBarAbort);
-    sh.epoch = ld_acquire_u32(q.bar + kBarEpoch);
-  }
-  if (warp == kOcWarps - 2 && lane == 0)
-    sh.lr = (p.flags & kFlagLrSchedule) ? 0.f : *p.d_lr;
-  if (warp == 8 && q.n_rounds > 0) load_pieces(sh.tab[0], q, 0, lane);
-  if (!kLars) {
-    step_constants<kNest, false>(p, &sh.unused_draw, &sh.skip, &sh.k, &sh.t);
-  } else if (threadIdx.x == 0) {
-    const int64_t t = p.d_step ? *p.d_step : int64_t(0);
-    sh.t = t;
-    sh.skip = 0;
-    sh.k = LambConsts{p.b1, p.omb1, p.b2, p.omb2, 1.f, 1.f, p.eps,
-                      0.f, 0.f, 0.f, 0.f};
-    if (blockIdx.x == 0) {
-      StepScalars sc{};
-      sc.t = t;
-      sc.c1 = 1.f;
-      sc.c2 = 1.f;
-      sc.lr = step_lr(p, t);
-      *p.scal = sc;
-    }
-  }
-  zero_red(sh);
-  __syncthreads();
-  // a launch after one that gave up does nothing more; a step count < 1 is
-  // skipped (status set by CTA 0)
-  if (sh.abort || sh.skip) return;
-  if (threadIdx.x == 0 && (p.flags & kFlagLrSchedule))
-    sh.lr = step_lr(p, sh.t);
-  if (q.n_rounds > 0) piece_rows(sh.tab[0]);
-  __syncthreads();
-  const LambConsts k = sh.k;
-  const float lr = sh.lr;
+  // ---- prologue (see the file header)
   const bool decoupled = !kLars && (p.flags & kFlagDecoupledDecay) != 0;
   const float wd = p.wd;
   const float coef = kLars ? (float)p.trust : 1.f;
-
-  if (q.n_rounds > 0) {
-    fused_pass<kOpt, GT, kCopy>(sh, s_rows, nullptr, &sh.tab[0], k, wd,
-                                decoupled);
-    __syncthreads();
+  zero_red(sh);
+  double mu_prod = 0.0;
+  if (warp >= kConstWarp) {
+    if (lane == 0) {
+      if (!kLars)
+        constants_part<kNest, false>(p, warp - kConstWarp, &sh.parts, nullptr);
+      else if (warp == kConstWarp)
+        sh.parts.t = p.d_step ? *p.d_step : int64_t(0);
+    }
+    __syncwarp();
+    asm volatile("bar.sync 1, %0;" :: "n"((kOcWarps - kConstWarp) * 32)
+                 : "memory");
+    if (threadIdx.x == kConstWarp * 32) {
+      if (kLars) {
+        sh.parts.skip = 0;
+        sh.k = LambConsts{p.b1, p.omb1, p.b2, p.omb2, 1.f, 1.f, p.eps,
+                          0.f, 0.f, 0.f, 0.f};
+      } else {
+        sh.k = constants_join<kNest>(p, sh.parts, &mu_prod);
+      }
+      if (p.flags & kFlagLrSchedule) sh.lr = step_lr(p, sh.parts.t);
+    }
+  } else {
+    if (warp == 1 && lane == 0) {
+      sh.abort = ld_acquire_u32(q.bar + kBarAbort);
+      sh.epoch = ld_acquire_u32(q.bar + kBarEpoch);
+    }
+    if (warp == 2 && lane == 0 && !(p.flags & kFlagLrSchedule))
+      sh.lr = *p.d_lr;
+    if (q.n_rounds > 0) {
+      if (warp == 0) load_pieces(sh.tab[0], q, 0, lane);
+      __syncwarp();
+      asm volatile("bar.sync 2, %0;" :: "n"(kConstWarp * 32) : "memory");
+      piece_rows(sh.tab[0]);
+      __syncwarp();
+      asm volatile("bar.sync 2, %0;" :: "n"(kConstWarp * 32) : "memory");
+    }
   }
+  // a launch after one that gave up does nothing; a step count < 1 is skipped
+  // (status set by CTA 0)
+  const bool go = fused_pass<kOpt, GT, kCopy>(
+      sh, s_rows, nullptr, q.n_rounds > 0 ? &sh.tab[0] : nullptr, wd,
+      decoupled, true);
+  const float lr = sh.lr;
+  if (blockIdx.x == 0 && threadIdx.x == kConstWarp * 32 && !sh.abort)
+    store_scalars(p, sh.parts.t, sh.parts.skip, lr, sh.k, mu_prod);
+  if (!go) return;
+  __syncthreads();
   for (int r = 0; r < q.n_rounds; ++r) {
     OcTables& T = sh.tab[r & 1];
     OcTables* next = r + 1 < q.n_rounds ? &sh.tab[(r + 1) & 1] : nullptr;
@@ -788,7 +812,7 @@ __global__ void __launch_bounds__(kOcThreads, 1)
     __syncthreads();
     if (!sh.ok) return;   // the launch gave up
     if (!next) finish_launch<kNest>(p, q, sh.epoch);
-    fused_pass<kOpt, GT, kCopy>(sh, s_rows, &T, next, k, wd, decoupled);
+    fused_pass<kOpt, GT, kCopy>(sh, s_rows, &T, next, wd, decoupled, false);
     __syncthreads();   // T's buffer is reloaded for round r + 2
   }
   if (q.n_rounds == 0) finish_launch<kNest>(p, q, sh.epoch);
