@@ -53,6 +53,11 @@ namespace {
 constexpr int kUnroll1 = 2;
 constexpr int kUnroll2 = 4;   // pass 2: 80 registers, 3 CTAs per SM
 constexpr int kMinBlocks1 = 3;
+// LARS reads and writes one state array less: 64 registers hold it, for
+// either type of g, so 4 CTAs run per SM.  ResNet-50, f32, the two launches:
+// 113.9 us at 80 registers and 3 CTAs, 110.8 us so (with the batches of the
+// norms' combine).
+constexpr int kMinBlocksLars1 = 4;
 
 // Sums of the first N of x[] over the CTA, valid in thread 0 (fixed trees:
 // lanes, then warps).  Contains one barrier; red must hold N rows.
@@ -76,8 +81,10 @@ __device__ __forceinline__ void cta_sum(float* x, float (*red)[kWarps]) {
 // fp64 combine of the chunk slots -> norms and trust ratio.  Thread t adds
 // slots t, t + kThreads, ... in that order; each warp adds its lanes, then
 // warp 0 the warps, in fixed trees.  Spreading the slots over the whole CTA
-// keeps a tensor of thousands of chunks (BERT's word embedding: 1,908) to a
-// few dependent L2 loads per thread.  Resets the ticket.  With the gradient
+// keeps a tensor of thousands of chunks (BERT's word embedding: 1,908) to
+// one batch of L2 loads per thread.  Resets the ticket.  What bounds it: load
+// latency, then fp64 issue (all 398 tensors of BERT-large in one launch:
+// 12.3 us with one load in flight and every warp in the trees, 8.8 us so).  With the gradient
 // check (kGn) it also forms the tensor's sum g^2 and whether any of its
 // elements was Inf/NaN, and counts the tensor done.
 template <bool kGn>
@@ -88,23 +95,48 @@ __device__ __noinline__ void finalize_tensor(const StepParams& p, int k,
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   double aw = 0.0, au = 0.0, ag = 0.0;
   float az = 0.f;
-  for (int i = (int)threadIdx.x; i < n; i += kThreads) {
-    const float2 s = __ldcg(&p.slots[first + i]);
-    aw += (double)s.x;
-    au += (double)s.y;
-    if (kGn) {
-      const float2 q = __ldcg(&p.grad_slots[first + i]);
-      ag += (double)q.x;
-      az += q.y;
-    }
-  }
+  // Where a thread has several slots, kFinBatch of them are in flight at
+  // once (a slot past the end adds an exact zero); the sums keep their
+  // order, and a warp without slots leaves its zeros as they are: fp64 adds
+  // are two a clock and SM here, so a whole CTA adding zeros shows.  The
+  // gradient check's four sums leave no registers for the batch (its step
+  // was 0.7% slower with it).
+  constexpr int kFinBatch = 8;
+  if (warp * 32 < n) {
+    int i = (int)threadIdx.x;
+    if (!kGn && n > kThreads) {
+      for (; i < n; i += kFinBatch * kThreads) {
+        float2 s[kFinBatch];
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    aw += __shfl_down_sync(0xffffffffu, aw, o);
-    au += __shfl_down_sync(0xffffffffu, au, o);
-    if (kGn) {
-      ag += __shfl_down_sync(0xffffffffu, ag, o);
-      az += __shfl_down_sync(0xffffffffu, az, o);
+        for (int j = 0; j < kFinBatch; ++j)
+          s[j] = i + j * kThreads < n
+                     ? __ldcg(&p.slots[first + i + j * kThreads])
+                     : make_float2(0.f, 0.f);
+#pragma unroll
+        for (int j = 0; j < kFinBatch; ++j) {
+          aw += (double)s[j].x;
+          au += (double)s[j].y;
+        }
+      }
+    }
+    for (; i < n; i += kThreads) {
+      const float2 s = __ldcg(&p.slots[first + i]);
+      aw += (double)s.x;
+      au += (double)s.y;
+      if (kGn) {
+        const float2 q = __ldcg(&p.grad_slots[first + i]);
+        ag += (double)q.x;
+        az += q.y;
+      }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      aw += __shfl_down_sync(0xffffffffu, aw, o);
+      au += __shfl_down_sync(0xffffffffu, au, o);
+      if (kGn) {
+        ag += __shfl_down_sync(0xffffffffu, ag, o);
+        az += __shfl_down_sync(0xffffffffu, az, o);
+      }
     }
   }
   if (lane == 0) {
@@ -128,9 +160,12 @@ __device__ __noinline__ void finalize_tensor(const StepParams& p, int k,
       az += __shfl_down_sync(0xffffffffu, az, o);
     }
   }
+  // both roots at once: lane 0's and lane 1's
+  const double au0 = __shfl_sync(0xffffffffu, au, 0);
+  const double wn = sqrt(lane == 1 ? au0 : aw);
+  const double un = __shfl_sync(0xffffffffu, wn, 1);
   int last_tensor = 0;
   if (lane == 0) {
-    const double wn = sqrt(aw), un = sqrt(au);
     double rho = 1.0;                                  // zero-norm rule
     if (!(wn == 0.0 || un == 0.0)) rho = coef * phi_of(wn, p) / un;
     p.ratio[k] = rho;
@@ -488,7 +523,7 @@ __device__ __forceinline__ void lars1_chunk(const TensorPtrs& tp,
 }
 
 template <typename GT, bool kGn>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, kGn ? kMinBlocks1 : kMinBlocksLars1)
     lars_pass1_kernel(const StepParams p) {
   __shared__ float red[4][kWarps];
   __shared__ uint32_t s_next[2];
