@@ -462,13 +462,15 @@ LAMB_API lamb_status_t lamb_layout_chunks(const int64_t* sizes, int32_t n_tensor
  * are rejected with LAMB_ERR_INVALID_ARG before any device work.  Calls no
  * cudaMalloc, cudaFree or other allocating routine.
  * The caller's host arrays (sizes, decay_mask and the five pointer arrays)
- * are copied into the device array with cudaMemcpyAsync on `stream`.  From
- * pageable memory those copies have read them when the call returns, so
- * they may be reused at once; from page-locked (pinned) memory a copy may
- * still be reading them after the call returns, so keep them unchanged until
- * `stream` has passed the call (e.g. synchronise it).  Under stream capture
- * the copies become graph nodes that read the same host arrays at every
- * replay, which must then stay valid and unchanged for the graph's life.
+ * travel with a kernel launch for up to 640 tensors: they have been read when
+ * the call returns, and a captured call keeps what it read.  Larger calls
+ * copy them into the device array with cudaMemcpyAsync on `stream`: from
+ * pageable memory those copies have read them when the call returns; from
+ * page-locked (pinned) memory a copy may still be reading them after the call
+ * returns, so keep them unchanged until `stream` has passed the call (e.g.
+ * synchronise it); and under stream capture the copies become graph nodes
+ * that read the same host arrays at every replay, which must then stay valid
+ * and unchanged for the graph's life.
  * The first call on each device (the current device) looks up the array's
  * device address; with CUDA's lazy module loading (the default) that first
  * use also loads the library's kernels and reserves the 4 MiB there, so make

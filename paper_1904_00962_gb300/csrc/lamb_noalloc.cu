@@ -105,23 +105,47 @@ cudaError_t na_setup(int dev, NaDevice** out) {
 }
 
 // ---- set-up kernel: builds the tables inside the scratch array -------------
-// One CTA of 1024 threads.  Reads the per-tensor sizes, mask and pointer
-// arrays the host copied into the scratch, and writes the tensor table,
-// pointer table (with the 128-bit alignment flag), tickets, default results
-// (ratio 1, norms 0), status and work counters; then every thread writes
-// every 1024th chunk of the chunk table, finding its tensor by a binary
-// search over the tensors' first chunks, kept in shared memory with the
-// length of each tensor's last chunk.
-constexpr int kSetupThreads = 1024;
-constexpr int kPerThread = kNaMaxTensors / kSetupThreads;   // 4
+// The caller's host arrays, for the tensors of one call.
+struct NaSource {
+  const int64_t* sizes;
+  const uint8_t* mask;      // NULL: every tensor decays
+  void* const* ptr[5];      // w, g, m, v, copy (NULL: no copies)
+};
 
-__global__ void __launch_bounds__(kSetupThreads)
-    noalloc_setup_kernel(int n, int has_mask, int grad_bf16, int has_v,
-                         int copy_bf16) {
+// The same arrays as a kernel parameter: up to kCap tensors go to the device
+// with the set-up launch itself.
+template <int kCap>
+struct NaArgs {
+  int64_t sizes[kCap];
+  void* ptr[5][kCap];
+  uint8_t mask[kCap];
+};
+// A launch takes at most 32764 bytes of parameters; a small step should not
+// carry all of them, so there are two sizes (161 tensors are a ResNet-50).
+constexpr int kNaArgsSmall = 192, kNaArgsLarge = 640;
+static_assert(sizeof(NaArgs<kNaArgsLarge>) + 16 <= 32764, "kernel parameters");
+
+// CTAs of 1024 threads.  Each scans the tensors' chunk counts for itself
+// (the first chunk and the last chunk's length of every tensor stay in its
+// shared memory); the tensors' tables (with the 128-bit alignment flag),
+// tickets and default results (ratio 1, norms 0) are written by whole warps
+// dealt over the CTAs, and every thread writes the chunk table's entries of
+// its grid-wide index, finding their tensor by a binary search.  The CTAs
+// share nothing, so none waits.
+//
+// What bounds it: latency -- the launch, the scan's few barriers and the
+// stores; hence one tensor a thread up to 1024 tensors, a scan by shuffles,
+// and kSetupChunks entries per CTA.  ResNet-50's 161 tensors and 1,643
+// chunks: 7.6 us by one CTA with a scan in shared memory, 5.9 us so; the
+// whole step 183 us with the arrays copied first, 173 us with the arrays in
+// the launch (its passes take 157 us of either).
+constexpr int kSetupThreads = 1024;
+constexpr int kSetupWarps = kSetupThreads / 32;
+constexpr int kSetupChunks = 256;
+
+__device__ __forceinline__ void build_tables(const NaSource& src, int n,
+                                             int grad_bf16) {
   unsigned char* s = g_noalloc_scratch;
-  const int64_t* sizes = reinterpret_cast<const int64_t*>(s + kOffSizes);
-  const uint8_t* mask = s + kOffMask;
-  void* const* raw = reinterpret_cast<void* const*>(s + kOffRaw);
   TensorDesc* tens = reinterpret_cast<TensorDesc*>(s + kOffTensors);
   TensorPtrs* ptrs = reinterpret_cast<TensorPtrs*>(s + kOffPtrs);
   ChunkDesc* chunks = reinterpret_cast<ChunkDesc*>(s + kOffChunks);
@@ -132,66 +156,73 @@ __global__ void __launch_bounds__(kSetupThreads)
   uint32_t* status = reinterpret_cast<uint32_t*>(s + kOffStatus);
   uint32_t* counters = reinterpret_cast<uint32_t*>(s + kOffCounters);
 
-  __shared__ int64_t part[kSetupThreads];
+  __shared__ int32_t s_warp[kSetupWarps];
   __shared__ int32_t s_first[kNaMaxTensors];     // first chunk of tensor k
   __shared__ int32_t s_lastlen[kNaMaxTensors];   // length of its last chunk
-  const int t = threadIdx.x;
-  // chunk counts of this thread's tensors, then an exclusive scan
-  int64_t local[kPerThread];
-  int64_t sum = 0;
-  for (int i = 0; i < kPerThread; ++i) {
-    const int k = t * kPerThread + i;
-    const int64_t d = k < n ? sizes[k] : 0;
-    local[i] = (d + kNaChunk - 1) / kNaChunk;
-    sum += local[i];
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  // thread t owns the tensors [t * per, (t + 1) * per)
+  const int per = (n + kSetupThreads - 1) / kSetupThreads;
+  int32_t sum = 0;              // at most kNaMaxChunks chunks in all
+  for (int i = 0; i < per; ++i) {
+    const int k = t * per + i;
+    if (k < n) sum += (int32_t)((src.sizes[k] + kNaChunk - 1) / kNaChunk);
   }
-  part[t] = sum;
+  int32_t incl = sum;           // inclusive scan in the warp, then of warps
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int32_t x = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += x;
+  }
+  if (lane == 31) s_warp[warp] = incl;
   __syncthreads();
-  for (int off = 1; off < kSetupThreads; off <<= 1) {   // Hillis-Steele
-    const int64_t x = t >= off ? part[t - off] : 0;
-    __syncthreads();
-    part[t] += x;
-    __syncthreads();
+  int32_t before = 0, n_chunks = 0;
+  for (int w = 0; w < kSetupWarps; ++w) {
+    const int32_t x = s_warp[w];
+    if (w < warp) before += x;
+    n_chunks += x;
   }
-  int64_t first = part[t] - sum;
-  for (int i = 0; i < kPerThread; ++i) {
-    const int k = t * kPerThread + i;
+  const bool mine = (uint32_t)warp % gridDim.x == blockIdx.x;
+  int32_t first = before + incl - sum;
+  for (int i = 0; i < per; ++i) {
+    const int k = t * per + i;
     if (k >= n) break;
-    const int64_t d = sizes[k];
-    TensorDesc td{};
-    td.numel = d;
-    td.first_chunk = (int32_t)first;
-    td.n_chunks = (int32_t)local[i];
-    td.decay = (!has_mask || mask[k]) ? 1.0f : 0.0f;
-    tens[k] = td;
-    s_first[k] = (int32_t)first;
-    s_lastlen[k] = (int32_t)(d - (local[i] - 1) * kNaChunk);
-    TensorPtrs tp{};
-    tp.w = static_cast<float*>(raw[0 * kNaMaxTensors + k]);
-    tp.g = raw[1 * kNaMaxTensors + k];
-    tp.m = static_cast<float*>(raw[2 * kNaMaxTensors + k]);
-    tp.v = has_v ? static_cast<float*>(raw[3 * kNaMaxTensors + k]) : nullptr;
-    tp.copy = copy_bf16 ? raw[4 * kNaMaxTensors + k] : nullptr;
-    const uintptr_t ga = grad_bf16 ? 8 : 16;
-    const bool ok = (uintptr_t)tp.w % 16 == 0 && (uintptr_t)tp.m % 16 == 0 &&
-                    (!tp.v || (uintptr_t)tp.v % 16 == 0) &&
-                    (uintptr_t)tp.g % ga == 0 &&
-                    (!tp.copy || (uintptr_t)tp.copy % 8 == 0);
-    tp.vec_ok = ok ? 1u : 0u;
-    ptrs[k] = tp;
-    first += local[i];
-    tickets[k] = 0u;
-    ratio[k] = 1.0;
-    wnorm[k] = 0.0;
-    unorm[k] = 0.0;
+    const int64_t d = src.sizes[k];
+    const int32_t nc = (int32_t)((d + kNaChunk - 1) / kNaChunk);
+    s_first[k] = first;
+    s_lastlen[k] = (int32_t)(d - (int64_t)(nc - 1) * kNaChunk);
+    if (mine) {
+      TensorDesc td{};
+      td.numel = d;
+      td.first_chunk = first;
+      td.n_chunks = nc;
+      td.decay = (!src.mask || src.mask[k]) ? 1.0f : 0.0f;
+      tens[k] = td;
+      TensorPtrs tp{};
+      tp.w = static_cast<float*>(src.ptr[0][k]);
+      tp.g = src.ptr[1][k];
+      tp.m = static_cast<float*>(src.ptr[2][k]);
+      tp.v = static_cast<float*>(src.ptr[3][k]);
+      tp.copy = src.ptr[4] ? src.ptr[4][k] : nullptr;
+      const uintptr_t ga = grad_bf16 ? 8 : 16;
+      const bool ok = (uintptr_t)tp.w % 16 == 0 && (uintptr_t)tp.m % 16 == 0 &&
+                      (uintptr_t)tp.v % 16 == 0 && (uintptr_t)tp.g % ga == 0 &&
+                      (uintptr_t)tp.copy % 8 == 0;
+      tp.vec_ok = ok ? 1u : 0u;
+      ptrs[k] = tp;
+      tickets[k] = 0u;
+      ratio[k] = 1.0;
+      wnorm[k] = 0.0;
+      unorm[k] = 0.0;
+    }
+    first += nc;
   }
-  if (t == 0) {
+  if (t == 0 && blockIdx.x == 0) {
     *status = 0u;
     counters[0] = counters[1] = counters[2] = counters[3] = 0u;
   }
-  __syncthreads();   // the tensor table is complete
-  const int32_t n_chunks = (int32_t)part[kSetupThreads - 1];
-  for (int32_t c = t; c < n_chunks; c += kSetupThreads) {
+  __syncthreads();   // the tensors' first chunks are complete
+  for (int32_t c = (int32_t)blockIdx.x + t * (int32_t)gridDim.x; c < n_chunks;
+       c += kSetupThreads * (int32_t)gridDim.x) {
     // the last tensor whose first chunk is <= c (a 0-chunk tensor shares its
     // first chunk with the next one, which comes later and wins)
     int lo = 0, hi = n - 1;
@@ -208,6 +239,71 @@ __global__ void __launch_bounds__(kSetupThreads)
     cd.len = c + 1 == end ? s_lastlen[lo] : kNaChunk;
     chunks[c] = cd;
   }
+}
+
+// The arrays come with the launch (at most kCap tensors).
+template <int kCap>
+__global__ void __launch_bounds__(kSetupThreads)
+    noalloc_setup_args_kernel(const __grid_constant__ NaArgs<kCap> a, int n,
+                              int has_mask, int grad_bf16, int copy_bf16) {
+  NaSource src;
+  src.sizes = a.sizes;
+  src.mask = has_mask ? a.mask : nullptr;
+  for (int i = 0; i < 4; ++i) src.ptr[i] = a.ptr[i];
+  src.ptr[4] = copy_bf16 ? a.ptr[4] : nullptr;
+  build_tables(src, n, grad_bf16);
+}
+
+// The arrays were copied into the scratch (any number of tensors).
+__global__ void __launch_bounds__(kSetupThreads)
+    noalloc_setup_kernel(int n, int has_mask, int grad_bf16, int copy_bf16) {
+  unsigned char* s = g_noalloc_scratch;
+  NaSource src;
+  src.sizes = reinterpret_cast<const int64_t*>(s + kOffSizes);
+  src.mask = has_mask ? s + kOffMask : nullptr;
+  for (int i = 0; i < 5; ++i)
+    src.ptr[i] = reinterpret_cast<void* const*>(s + kOffRaw) +
+                 (size_t)i * kNaMaxTensors;
+  if (!copy_bf16) src.ptr[4] = nullptr;
+  build_tables(src, n, grad_bf16);
+}
+
+// The caller's arrays, as the host sees them.
+struct NaHost {
+  const int64_t* sizes;
+  const uint8_t* mask;
+  const void* const* ptr[5];
+};
+
+template <int kCap>
+cudaError_t setup_from_args(const NaHost& a, int n, int grad_bf16, int grid,
+                            cudaStream_t stream) {
+  NaArgs<kCap> args;   // the launch copies it; entries past n are not read
+  std::memcpy(args.sizes, a.sizes, (size_t)n * 8);
+  for (int i = 0; i < 5; ++i)
+    if (a.ptr[i]) std::memcpy(args.ptr[i], a.ptr[i], (size_t)n * 8);
+  if (a.mask) std::memcpy(args.mask, a.mask, (size_t)n);
+  noalloc_setup_args_kernel<kCap><<<grid, kSetupThreads, 0, stream>>>(
+      args, n, a.mask ? 1 : 0, grad_bf16, a.ptr[4] ? 1 : 0);
+  return cudaGetLastError();
+}
+
+cudaError_t setup_from_copies(unsigned char* s, const NaHost& a, int n,
+                              int grad_bf16, int grid, cudaStream_t stream) {
+  const size_t nb = (size_t)n * 8;
+  cudaError_t e = cudaMemcpyAsync(s + kOffSizes, a.sizes, nb,
+                                  cudaMemcpyHostToDevice, stream);
+  if (e == cudaSuccess && a.mask)
+    e = cudaMemcpyAsync(s + kOffMask, a.mask, (size_t)n,
+                        cudaMemcpyHostToDevice, stream);
+  for (int i = 0; i < 5 && e == cudaSuccess; ++i)
+    if (a.ptr[i])
+      e = cudaMemcpyAsync(s + kOffRaw + (size_t)i * 8 * kNaMaxTensors,
+                          a.ptr[i], nb, cudaMemcpyHostToDevice, stream);
+  if (e != cudaSuccess) return e;
+  noalloc_setup_kernel<<<grid, kSetupThreads, 0, stream>>>(
+      n, a.mask ? 1 : 0, grad_bf16, a.ptr[4] ? 1 : 0);
+  return cudaGetLastError();
 }
 
 }  // namespace
@@ -294,26 +390,22 @@ extern "C" LAMB_API lamb_status_t lamb_step_noalloc(
                    cudaGetErrorString(e));
   unsigned char* s = nd->scratch;
 
-  // ---- stage the caller's host arrays into the scratch ---------------------
-  const size_t nb = (size_t)n_tensors * 8;
-  e = cudaMemcpyAsync(s + kOffSizes, sizes, nb, cudaMemcpyHostToDevice, stream);
-  if (e == cudaSuccess && decay_mask)
-    e = cudaMemcpyAsync(s + kOffMask, decay_mask, (size_t)n_tensors,
-                        cudaMemcpyHostToDevice, stream);
-  const void* const* arrays[5] = {w, g, m, v, copy ? w_copy : nullptr};
-  for (int i = 0; i < 5 && e == cudaSuccess; ++i)
-    if (arrays[i])
-      e = cudaMemcpyAsync(s + kOffRaw + (size_t)i * 8 * kNaMaxTensors,
-                          arrays[i], nb, cudaMemcpyHostToDevice, stream);
+  // ---- the tables, from the caller's host arrays ---------------------------
+  // As a parameter of the set-up launch as far as they fit: one launch in
+  // place of six or seven copies and a launch.
+  const int gbf = grad_dtype == LAMB_BF16 ? 1 : 0;
+  const NaHost host = {sizes, decay_mask, {w, g, m, v, copy ? w_copy : nullptr}};
+  int sgrid = (int)((n_chunks + kSetupChunks - 1) / kSetupChunks);
+  if (sgrid > nd->num_sms) sgrid = nd->num_sms;
+  if (sgrid < 1) sgrid = 1;
+  if (n_tensors <= kNaArgsSmall)
+    e = setup_from_args<kNaArgsSmall>(host, n_tensors, gbf, sgrid, stream);
+  else if (n_tensors <= kNaArgsLarge)
+    e = setup_from_args<kNaArgsLarge>(host, n_tensors, gbf, sgrid, stream);
+  else
+    e = setup_from_copies(s, host, n_tensors, gbf, sgrid, stream);
   if (e != cudaSuccess)
-    return na_fail(LAMB_ERR_CUDA, "lamb_step_noalloc: staging copy: %s",
-                   cudaGetErrorString(e));
-  noalloc_setup_kernel<<<1, kSetupThreads, 0, stream>>>(
-      n_tensors, decay_mask ? 1 : 0, grad_dtype == LAMB_BF16 ? 1 : 0, 1,
-      copy ? 1 : 0);
-  e = cudaGetLastError();
-  if (e != cudaSuccess)
-    return na_fail(LAMB_ERR_CUDA, "lamb_step_noalloc: set-up launch: %s",
+    return na_fail(LAMB_ERR_CUDA, "lamb_step_noalloc: set-up: %s",
                    cudaGetErrorString(e));
 
   // ---- the two LAMB passes on tables inside the scratch --------------------
@@ -337,7 +429,6 @@ extern "C" LAMB_API lamb_status_t lamb_step_noalloc(
   sp.d_step = d_step;
   sp.d_lr = d_lr;
   sp.n_chunks = (int32_t)n_chunks;
-  const int gbf = grad_dtype == LAMB_BF16 ? 1 : 0;
   auto grid_of = [&](int occ) {
     int64_t gsz = (int64_t)nd->num_sms * (occ < 1 ? 1 : occ);
     if (gsz > n_chunks) gsz = n_chunks;
@@ -348,7 +439,7 @@ extern "C" LAMB_API lamb_status_t lamb_step_noalloc(
     rc = launch_lamb_pass2(sp, 0, gbf, copy ? 1 : 0,
                            grid_of(nd->occ[2 + (copy ? 1 : 0)]), stream);
   if (!rc && d_ratio)
-    rc = (int)cudaMemcpyAsync(d_ratio, s + kOffRatio, nb,
+    rc = (int)cudaMemcpyAsync(d_ratio, s + kOffRatio, (size_t)n_tensors * 8,
                               cudaMemcpyDeviceToDevice, stream);
   if (rc)
     return na_fail(LAMB_ERR_CUDA, "lamb_step_noalloc: %s",
