@@ -129,6 +129,25 @@ def kernel_model(opt, algo, gb, cb, variant="plain", streamed_frac=0.0):
     return names, [gb + 12 + 8, 12 + (gb if nest else 0) + 4 + cb]
 
 
+def one_launch_model(opt, gb, cb, variant="plain"):
+    """kernel_model of the one-launch form of a step: every operand once
+    (tensors too large to be kept are read again in part, which is not
+    counted).  The gradient check and the skip mode read g first."""
+    names = [f"stash_step_kernel<{opt},g{8 * gb},copy{8 * cb}>"]
+    per = [single_touch_bytes(opt, gb, cb)]
+    if variant in ("grad_norm", "skip_nonfinite"):
+        return [f"grad_check_kernel<g{8 * gb}>"] + names, [gb] + per
+    return names, per
+
+
+def one_launch_on_chip_plan(sizes, n_rounds):
+    """AUTO's rule for an on-chip plan of several rounds: three rounds or
+    more and chunks (10,240 elements at most) of 5,400 elements on average
+    step in one launch over all tensors instead of round by round."""
+    chunks = sum(-(-s // 10240) for s in sizes)
+    return n_rounds >= 3 and sum(sizes) >= 5400 * chunks
+
+
 def noalloc_overhead(st, L, hyper, d_step, d_lr, stream, one_step, n=20):
     """Device time and host enqueue time per call of lamb_step_noalloc
     against the plan's lamb_step, on the same state, n calls each after
@@ -674,13 +693,22 @@ def run_ours(args):
     ms_instr = e0.elapsed_time(e1)
     n_timed, ms_kernels = B.lamb_plan_read_timing(plan.handle, 3)
     B.lamb_plan_set_timing(plan.handle, False)
-    if algo == 1 and sum(ms > 0 for ms in ms_kernels) == 1:
-        # a two-pass plan's one-launch form: every operand once (tensors too
-        # large to be kept are read again in part, which is not counted)
-        gb = 2 if L.grad_dtype == "bf16" else 4
-        cb = 2 if L.copy_dtype == "bf16" else 0
-        kernel_names = [f"stash_step_kernel<{opt},g{8 * gb},copy{8 * cb}>"]
-        kernel_bytes, profile = [single_touch_bytes(opt, gb, cb)], None
+    # AUTO's one-launch form: a plain step of a two-pass plan is then one
+    # kernel; an on-chip plan's step is one kernel either way
+    B.lamb_plan_set_timing(plan.handle, True)
+    plan.step_call(opt, layout_hyper(L, opt, "plain")[1], d_step, d_lr,
+                   d_prod if opt in ("nlamb", "nnlamb") else None, 0.004,
+                   stream)()
+    barrier()
+    n_plain = sum(ms > 0 for ms in B.lamb_plan_read_timing(plan.handle, 3)[1])
+    B.lamb_plan_set_timing(plan.handle, False)
+    if args.algo == "auto" and n_plain == 1 and (
+            algo == 1 or (opt != "lars" and one_launch_on_chip_plan(
+                L.sizes, info["n_rounds"]))):
+        kernel_names, kernel_bytes = one_launch_model(
+            opt, 2 if L.grad_dtype == "bf16" else 4,
+            2 if L.copy_dtype == "bf16" else 0, args.variant)
+        profile = None
     # The first K timed steps are the measurement.  When the two regions take
     # less than CLOCK_WINDOW_S, the same K-step region runs again (each timed
     # the same way) until the clock sampler has watched the GPU for that long,
