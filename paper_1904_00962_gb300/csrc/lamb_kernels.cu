@@ -40,6 +40,7 @@
 #include <type_traits>
 
 #include "lamb_device.cuh"
+#include "lamb_sync.cuh"
 
 namespace lamb {
 namespace {
@@ -313,6 +314,8 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks1)
   __shared__ uint32_t s_next[2];
   __shared__ int s_last, s_skip;
   __shared__ LambConsts s_k;
+  // (a sharded pass 1 is followed by the caller's own work)
+  if (!(p.flags & kFlagNoFinalize)) let_next_launch();
   step_constants<kNest, true>(p, s_next, &s_skip, &s_k, nullptr);
   if (s_skip) return;
   const LambConsts k = s_k;
@@ -425,6 +428,7 @@ template <bool kCopy, int kNest, typename GT, bool kDefer>
 __global__ void __launch_bounds__(kThreads)
     lamb_pass2_kernel(const StepParams p) {
   __shared__ uint32_t s_next[2];
+  after_prior_launch();
   const StepScalars sc = *p.scal;
   if (sc.skip) return;
   // a step whose gradients held an Inf/NaN writes nothing (and does not
@@ -528,6 +532,7 @@ __global__ void __launch_bounds__(kThreads, kGn ? kMinBlocks1 : kMinBlocksLars1)
   __shared__ float red[4][kWarps];
   __shared__ uint32_t s_next[2];
   __shared__ int s_last;
+  if (!(p.flags & kFlagNoFinalize)) let_next_launch();
   if (threadIdx.x == 0) {
     if (blockIdx.x == 0) {
       StepScalars sc{};
@@ -622,6 +627,7 @@ template <bool kCopy, typename GT, bool kDefer>
 __global__ void __launch_bounds__(kThreads)
     lars_pass2_kernel(const StepParams p) {
   __shared__ uint32_t s_next[2];
+  after_prior_launch();
   const StepScalars sc = *p.scal;
   if (kDefer && p.gcheck->nonfinite) return;   // skipped step: no writes
   if (threadIdx.x == 0) s_next[0] = atomicAdd(&p.counters[1], 1u);
@@ -650,12 +656,36 @@ __global__ void __launch_bounds__(kThreads)
 __global__ void __launch_bounds__(kThreads)
     finalize_all_kernel(const StepParams p, double coef) {
   // one CTA per tensor, as when pass 1 finalises it: the same sums
+  let_next_launch();
   for (int k = (int)blockIdx.x; k < p.n_tensors; k += (int)gridDim.x) {
     const TensorDesc td = p.tensors[k];
     if (td.n_chunks > 0)
       finalize_tensor<false>(p, k, td.first_chunk, td.n_chunks, coef);
     __syncthreads();   // the finaliser's shared sums are reused
   }
+}
+
+// kernel<<<grid, kThreads>>>(p), allowed to start before the launch in front
+// of it on the stream has ended: only for a kernel that calls
+// after_prior_launch() first, and only behind a launch of this library that
+// itself came after everything older on the stream (the wait covers that one
+// launch, not what an early-started caller's kernel may have left running).
+// It saves the gap between the two launches, 2 us per pair: ResNet-50 LARS
+// 110.8 -> 109.2 us, one of eight shards of BERT-large 279.0 -> 276.0 us.
+int launch_after(void (*kernel)(const StepParams), const StepParams& p,
+                 int grid, cudaStream_t s) {
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3(kThreads);
+  cfg.stream = s;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, p);
+  if (e != cudaSuccess) (void)cudaGetLastError();   // reported here, once
+  return (int)e;
 }
 
 template <typename K>
@@ -679,10 +709,8 @@ int lamb_p2(const StepParams& p, int grid, cudaStream_t s) {
   // plain LAMB's pass 2 does not read g: one instantiation for both types
   using GT2 = typename std::conditional<kNest != 0, GT, float>::type;
   if (p.flags & kFlagSkipNonfinite)
-    lamb_pass2_kernel<kCopy, kNest, GT, true><<<grid, kThreads, 0, s>>>(p);
-  else
-    lamb_pass2_kernel<kCopy, kNest, GT2, false><<<grid, kThreads, 0, s>>>(p);
-  return (int)cudaGetLastError();
+    return launch_after(lamb_pass2_kernel<kCopy, kNest, GT, true>, p, grid, s);
+  return launch_after(lamb_pass2_kernel<kCopy, kNest, GT2, false>, p, grid, s);
 }
 
 template <typename GT>
@@ -697,10 +725,8 @@ int lars_p1(const StepParams& p, int grid, cudaStream_t s) {
 template <bool kCopy, typename GT>
 int lars_p2(const StepParams& p, int grid, cudaStream_t s) {
   if (p.flags & kFlagSkipNonfinite)
-    lars_pass2_kernel<kCopy, GT, true><<<grid, kThreads, 0, s>>>(p);
-  else
-    lars_pass2_kernel<kCopy, float, false><<<grid, kThreads, 0, s>>>(p);
-  return (int)cudaGetLastError();
+    return launch_after(lars_pass2_kernel<kCopy, GT, true>, p, grid, s);
+  return launch_after(lars_pass2_kernel<kCopy, float, false>, p, grid, s);
 }
 
 }  // namespace

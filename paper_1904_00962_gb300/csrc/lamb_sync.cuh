@@ -1,12 +1,24 @@
-// PTX helpers of the kernels whose CTAs exchange data while they run
-// (lamb_onchip.cu, lamb_stash.cu): scoped loads and stores, the global
-// timer, mbarriers, and tensor memory used as per-warp storage.
+// PTX helpers: launches that follow one another early (lamb_kernels.cu), and
+// for the kernels whose CTAs exchange data while they run (lamb_onchip.cu,
+// lamb_stash.cu) scoped loads and stores, the global timer, mbarriers, and
+// tensor memory used as per-warp storage.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
 
 namespace lamb {
 namespace {
+
+// Two launches in a row: the second may be launched while the first still
+// runs; its CTAs start as the first one's leave, and wait in
+// after_prior_launch() until the first one has ended and its writes are
+// visible.  A kernel launched the ordinary way passes the wait at once.
+__device__ __forceinline__ void after_prior_launch() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ void let_next_launch() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
 
 __device__ __forceinline__ uint32_t ld_acquire_u32(const uint32_t* p) {
   uint32_t v;

@@ -114,3 +114,54 @@ def test_noalloc_tables_of_many_tensors_match_the_plan(n, mask):
         assert torch.equal(x, y), name
     assert torch.equal(ratio, plan.results()[0])
     plan.destroy()
+
+
+@pytest.mark.parametrize("opt", ["lamb", "lars", "noalloc"])
+def test_captured_passes_replay_like_eager_steps(opt):
+    """The second pass starts behind the first before it has ended: five
+    steps in a row, eager and replayed, on many small tensors (the first pass
+    ends late) and one of 2,000 chunks."""
+    sizes = [1 + (97 * k) % 5000 for k in range(300)] + [16384 * 2000 + 3]
+    out = []
+    for captured in (False, True):
+        st = DeviceState(sizes)
+        gen = torch.Generator(device="cuda:0")
+        gen.manual_seed(9)
+        for name, scale in (("w", 0.02), ("g", 1e-3), ("m", 1e-3),
+                            ("v", 1e-6)):
+            t = torch.randn(getattr(st, name).numel(), device="cuda:0",
+                            generator=gen) * scale
+            getattr(st, name).copy_(t.abs() if name == "v" else t)
+        step, lr = _scalars()
+        hyper = B.make_hyper(increment_step=True, bias_correction=opt != "lars",
+                             trust_coef=1e-2 if opt == "lars" else 1.0)
+        plan = LambPlan(st, algorithm=B.LAMB_ALGO_TWO_PASS)
+        ptrs = [st.ptrs(x) for x in ("w", "g", "m", "v")]
+
+        def one():
+            if opt == "lamb":
+                plan.lamb_step(hyper, step, lr)
+            elif opt == "lars":
+                plan.lars_step(hyper, step, lr)
+            else:
+                B.lamb_step_noalloc(sizes, None, B.LAMB_F32,
+                                    B.LAMB_DTYPE_NONE, *ptrs, None, hyper,
+                                    step.data_ptr(), lr.data_ptr(), 0,
+                                    torch.cuda.current_stream().cuda_stream)
+        one()
+        torch.cuda.synchronize()
+        if captured:
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph):
+                one()
+            for _ in range(5):
+                graph.replay()
+        else:
+            for _ in range(5):
+                one()
+        torch.cuda.synchronize()
+        assert int(step.item()) == 3 + 6
+        out.append([getattr(st, x).clone() for x in ("w", "m", "v")])
+        plan.destroy()
+    for a, b in zip(*out):
+        assert torch.equal(a, b)
