@@ -25,7 +25,8 @@
  * g is float32 or bfloat16; an optional bfloat16 copy of the new w is written
  * with round-to-nearest-even.  All tensor pointers are DEVICE pointers on the
  * plan's device.  Pointers aligned to 16 bytes (8 bytes for bfloat16 arrays)
- * take the vectorised path; others are handled element by element.
+ * take the vectorised path; others are handled element by element (AUTO's
+ * one-launch steps stream them in whole 16-byte granules all the same).
  *
  * Ownership: the caller owns w, g, m, v, the bf16 copy, the step counter,
  * the learning rate and the streams.  The plan owns its chunk table, pointer
@@ -100,7 +101,9 @@ typedef enum { LAMB_PHI_IDENTITY = 0, LAMB_PHI_CLIP = 1 } lamb_phi_t;
                                            across chunks: a chunk whose sum
                                            of g^2 exceeds FLT_MAX reports an
                                            infinite norm without counting as
-                                           non-finite                       */
+                                           non-finite.  A plan that AUTO lets
+                                           step in one launch reads g in a
+                                           launch of its own first          */
 #define LAMB_FLAG_SKIP_NONFINITE  0x10u /* implies GRAD_NORM.  If any element
                                            of g is Inf or NaN the step writes
                                            nothing: w, m, v, the bf16 copy,
@@ -109,7 +112,8 @@ typedef enum { LAMB_PHI_IDENTITY = 0, LAMB_PHI_CLIP = 1 } lamb_phi_t;
                                            values, and LAMB_STATUS_SKIPPED is
                                            set.  Pass 2 then forms and writes
                                            m, v instead of pass 1: one more
-                                           read of g per step              */
+                                           read of g per step (by the launch
+                                           in front on a one-launch plan)  */
 #define LAMB_FLAG_DECOUPLED_DECAY 0x20u /* lamb_step / nlamb_step only: the
                                            decay term leaves the normalised
                                            direction, u = r, rho = phi(||w||)
@@ -167,11 +171,13 @@ typedef struct {
                                      the two-pass kernels
                                      (lamb_plan_get_info reports the choice).
                                      A two-pass plan made by AUTO runs its
-                                     steps without the gradient check as ONE
-                                     launch where most of the layout fits the
-                                     SMs in turn: a chunk's w and u stay on
-                                     the SM until its tensor's ratio is known
-                                     (28 B of HBM traffic per parameter).  m,
+                                     steps as ONE launch (behind one that
+                                     reads g, with the gradient check or the
+                                     skip mode) where most of the layout fits
+                                     the SMs in turn: a chunk's w and u stay
+                                     on the SM until its tensor's ratio is
+                                     known (28 B of HBM traffic per
+                                     parameter).  m,
                                      v and u are the two kernels' bit for bit;
                                      the norms are summed in another fixed
                                      order.  So does an on-chip plan made
@@ -196,7 +202,7 @@ typedef struct {
                                      then).  LAMB, LARS, N-LAMB, NN-LAMB,
                                      decoupled decay and the schedule; the
                                      gradient check and the skip mode run
-                                     two-pass on such a plan               */
+                                     two-pass on such a plan (AUTO's: above) */
 #define LAMB_ONCHIP_ROW_ELEMS 128
 #define LAMB_TAIL_CHUNK_ELEMS 2048
 

@@ -66,9 +66,11 @@ size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 }  // namespace
 
-// LAMB_ALGO_AUTO takes the on-chip step up to this many rounds (measured:
-// ResNet-50, 7 rounds, 5.7% faster on-chip; the ragged layout, 623 rounds,
-// 4.5% slower).
+// LAMB_ALGO_AUTO makes an on-chip plan up to this many rounds, a two-pass plan
+// beyond (two launches against the on-chip kernel: ResNet-50, 7 rounds, 5.7%
+// slower; the ragged layout, 623 rounds, 4.5% faster).  From three rounds on
+// most LAMB steps of either plan run as one launch (below); the line decides
+// what lamb_plan_get_info reports and what the other steps run.
 constexpr int kAutoMaxRounds = 32;
 
 // An AUTO on-chip plan's steps take the one-launch form of the two-pass step
@@ -863,11 +865,12 @@ static void fill_params(lamb_plan* p, const lamb_hyper_t* h, int64_t* d_step,
   }
 }
 
-// The on-chip kernel runs every step but those with the gradient check or the
-// skip mode (their decision needs all of g before anything is written), and,
-// on a plan that AUTO made on-chip, LARS steps over several rounds: LARS's
-// two-pass step moves only 8 B/parameter more, less than the per-round cost
-// of the on-chip exchange (ResNet-50: 0.111 against 0.120 ms).
+// An on-chip plan's steps leave the two-pass path here, but for those with the
+// gradient check or the skip mode (their decision needs all of g before
+// anything is written), and, on a plan that AUTO made on-chip, LARS steps over
+// several rounds: LARS's two-pass step moves only 8 B/parameter more, less
+// than the per-round cost of the on-chip exchange (ResNet-50: 109 against 114
+// us).
 static bool onchip_takes(const lamb_plan* p, uint32_t flags, bool lars) {
   return p->algorithm == LAMB_ALGO_ON_CHIP &&
          !(flags & (LAMB_FLAG_GRAD_NORM | LAMB_FLAG_SKIP_NONFINITE)) &&
