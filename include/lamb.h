@@ -173,7 +173,8 @@ typedef struct {
                                      A two-pass plan made by AUTO runs its
                                      steps as ONE launch (behind one that
                                      reads g, with the gradient check or the
-                                     skip mode) where most of the layout fits
+                                     skip mode; lars_step with either keeps
+                                     the two kernels) where most of the layout fits
                                      the SMs in turn: a chunk's w and u stay
                                      on the SM until its tensor's ratio is
                                      known (28 B of HBM traffic per

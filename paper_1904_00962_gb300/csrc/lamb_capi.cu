@@ -927,10 +927,13 @@ static int launch_onchip_step(const lamb_plan* p, const StepParams& sp,
 // two launches' rate (one launch / two, us: 200 tensors of 1M, none again, LAMB
 // 877 / 1207, LARS 694 / 827; one of 10M, 0.4 again, 73 / 85 and 62 / 63; 40 of
 // 8M, 0.45 again, 1950 / 1914 and 1648 / 1313; one of 30M, 0.8 again, 209 / 205
-// and 176 / 143).
-static bool stash_takes(const lamb_plan* p, bool lars) {
+// and 176 / 143).  LARS has 8 B/parameter to win and the check's read of g
+// takes 2 or 4 of them: with it the two launches stay (76.8M parameters in 161
+// tensors, bf16 g: 335 in one launch behind the check, 304 in two).
+static bool stash_takes(const lamb_plan* p, uint32_t flags, bool lars) {
   return p->st_grid > 0 &&
          !(lars && p->algorithm == LAMB_ALGO_ON_CHIP) &&
+         !(lars && (flags & (LAMB_FLAG_GRAD_NORM | LAMB_FLAG_SKIP_NONFINITE))) &&
          p->st_again <= (lars ? 0.2 : 0.4);
 }
 
@@ -941,7 +944,7 @@ static int launch_two_pass_step(const lamb_plan* p, const StepParams& sp,
                                 cudaEvent_t* ev) {
   const bool lars = opt == 3;
   int rc = 0;
-  if (stash_takes(p, lars)) {
+  if (stash_takes(p, sp.flags, lars)) {
     StashParams q;
     q.recs = p->st_recs;
     q.words = p->st_words;
@@ -998,7 +1001,7 @@ static lamb_status_t launch_step(lamb_plan* p, const StepParams& sp, int opt,
     const cudaError_t e = cudaEventRecord(ev[0], stream);
     if (e != cudaSuccess) return cuda_fail(e, what);
   }
-  const int n = !stash_takes(p, opt == 3) &&
+  const int n = !stash_takes(p, sp.flags, opt == 3) &&
                         onchip_takes(p, sp.flags, opt == 3)
                     ? launch_onchip_step(p, sp, opt, stream, ev)
                     : launch_two_pass_step(p, sp, opt, stream, ev);

@@ -176,6 +176,20 @@ def test_gradient_check_matches_the_two_pass_kernels(opt, grad, copy, misalign,
         np.testing.assert_allclose(a.cpu(), b.cpu(), rtol=2 * TOL_RATIO)
 
 
+@pytest.mark.parametrize("flag", ["grad_norm", "skip_nonfinite"])
+def test_lars_with_the_gradient_check_keeps_the_two_kernels(flag):
+    """Bit for bit, norms included: their sums' order, not the launch's."""
+    outs = []
+    for algo in (B.LAMB_ALGO_AUTO, B.LAMB_ALGO_TWO_PASS):
+        r = Run(SIZES, opt="lars", flags={flag: True}, algorithm=algo,
+                onchip_max_ctas=5)
+        r.step()
+        a, b = r.out()
+        outs.append(a + b)
+        r.plan.destroy()
+    assert _same(*outs)
+
+
 def test_gradient_check_of_a_step_with_a_bad_count_does_nothing():
     r = Run(SIZES, flags={"skip_nonfinite": True}, onchip_max_ctas=5)
     r.st.view("g", 20)[5] = float("nan")
