@@ -65,6 +65,9 @@ ALGO_CODES = {"auto": 0, "two_pass": 1, "on_chip": 3}
 TWO_PASS_SOURCES = ("lamb_kernels.cu", "lamb_device.cuh", "lamb_internal.h")
 ONCHIP_SOURCES = ("lamb_onchip.cu", "lamb_onchip.h", "lamb_device.cuh",
                   "lamb_internal.h")
+STASH_SOURCES = ("lamb_stash.cu", "lamb_stash.h", "lamb_sync.cuh",
+                 "lamb_device.cuh", "lamb_internal.h")
+STASH_PROFILE = os.path.join(ROOT, "profiles", "stash_step_kernel.md")
 PROFILES = {
     (1, "bert_large", "lamb"): (
         os.path.join(ROOT, "profiles", "lamb_kernels_bert_large.md"),
@@ -702,13 +705,15 @@ def run_ours(args):
     barrier()
     n_plain = sum(ms > 0 for ms in B.lamb_plan_read_timing(plan.handle, 3)[1])
     B.lamb_plan_set_timing(plan.handle, False)
-    if args.algo == "auto" and n_plain == 1 and (
+    lars_check = lars and args.variant in ("grad_norm", "skip_nonfinite")
+    if args.algo == "auto" and n_plain == 1 and not lars_check and (
             algo == 1 or (opt != "lars" and one_launch_on_chip_plan(
                 L.sizes, info["n_rounds"]))):
         kernel_names, kernel_bytes = one_launch_model(
             opt, 2 if L.grad_dtype == "bf16" else 4,
             2 if L.copy_dtype == "bf16" else 0, args.variant)
-        profile = None
+        profile = (STASH_PROFILE, f"{args.layout}/{opt}", STASH_SOURCES) if (
+            args.variant == "plain" and args.layers == 24) else None
     # The first K timed steps are the measurement.  When the two regions take
     # less than CLOCK_WINDOW_S, the same K-step region runs again (each timed
     # the same way) until the clock sampler has watched the GPU for that long,
