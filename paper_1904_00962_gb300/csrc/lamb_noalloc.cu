@@ -138,7 +138,7 @@ static_assert(sizeof(NaArgs<kNaArgsLarge>) + 16 <= 32764, "kernel parameters");
 // and kSetupChunks entries per CTA.  ResNet-50's 161 tensors and 1,643
 // chunks: 7.6 us by one CTA with a scan in shared memory, 5.9 us so; the
 // whole step 183 us with the arrays copied first, 173 us with the arrays in
-// the launch (its passes take 157 us of either).
+// the launch (171 since pass 2 is launched early; the passes take 157).
 constexpr int kSetupThreads = 1024;
 constexpr int kSetupWarps = kSetupThreads / 32;
 constexpr int kSetupChunks = 256;
