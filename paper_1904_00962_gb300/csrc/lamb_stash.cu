@@ -145,6 +145,17 @@ __device__ __forceinline__ bool wait_phase(const Shared& sh, uint64_t* b,
     if (aborted(sh)) return false;
   return true;
 }
+// The same, and whether the launch gives up, with one answer for a warp: its
+// lanes look at the flag one by one, and lanes that left alone would be waited
+// for in the next warp-wide operation.
+constexpr uint32_t kAllLanes = 0xffffffffu;
+__device__ __forceinline__ bool warp_wait(const Shared& sh, uint64_t* b,
+                                          uint32_t parity) {
+  return __all_sync(kAllLanes, wait_phase(sh, b, parity));
+}
+__device__ __forceinline__ bool warp_aborted(const Shared& sh) {
+  return __any_sync(kAllLanes, aborted(sh));
+}
 __device__ __forceinline__ uint32_t phase_of(int seq) {
   return (uint32_t)(seq / kStashRecs) & 1u;
 }
@@ -291,16 +302,14 @@ struct Worker {
   }
 
   __device__ __forceinline__ bool all_test(uint64_t* b, uint32_t parity) {
-    return __all_sync(0xffffffffu, mbar_test(b, parity));
+    return __all_sync(kAllLanes, mbar_test(b, parity));
   }
   __device__ __forceinline__ bool head_ready() {
     return hseq < kseq &&
            all_test(&sh.kready[hseq % kStashRecs], phase_of(hseq));
   }
   __device__ __forceinline__ bool head_wait() {
-    return __all_sync(0xffffffffu,
-                      wait_phase(sh, &sh.kready[hseq % kStashRecs],
-                                 phase_of(hseq)));
+    return warp_wait(sh, &sh.kready[hseq % kStashRecs], phase_of(hseq));
   }
 
   // Where slot x has its u, and its w if that is in tensor memory.
@@ -484,7 +493,7 @@ struct Worker {
     while (!all_test(b, parity)) {
       if (head_ready())
         update_some();
-      else if (aborted(sh))
+      else if (warp_aborted(sh))
         return false;
       else
         __nanosleep(32);
@@ -620,20 +629,22 @@ __device__ __forceinline__ void draw(const StepParams& p, const StashParams& q,
   for (int seq = 0;; ++seq) {
     const int slot = seq % kStashRecs;
     if (seq >= kStashRecs &&
-        !wait_phase(sh, &sh.free[slot], phase_of(seq - kStashRecs)))
+        !warp_wait(sh, &sh.free[slot], phase_of(seq - kStashRecs)))
       return;
-    __syncwarp();
     // Drawn only when all that was drawn before is on its way in: work that a
     // CTA holds while its ring is full delays its tensor for every other CTA
     // (BERT-large, drawing 0 / 2 / 6 tiles early: 1503 / 1570 / 1632 us).
-    while (drawn - *reinterpret_cast<volatile int*>(&sh.issued) > 0) {
-      if (aborted(sh)) return;
+    while (__any_sync(kAllLanes,
+                      drawn - *reinterpret_cast<volatile int*>(&sh.issued) >
+                          0)) {
+      if (warp_aborted(sh)) return;
       __nanosleep(32);
     }
     // a CTA full of one tensor's chunks draws no more of them
     if (kept >= q.max_keep) {
-      while ((int)ld_relaxed_u32(q.bar + kStashCounter) < keep_end) {
-        if (aborted(sh)) return;
+      while (__any_sync(kAllLanes, (int)ld_relaxed_u32(q.bar + kStashCounter) <
+                                       keep_end)) {
+        if (warp_aborted(sh)) return;
         __nanosleep(100);
       }
     }
@@ -670,7 +681,7 @@ __device__ __forceinline__ void draw(const StepParams& p, const StashParams& q,
     const int n = chunk_tiles(len, (bits & kStashVec) != 0);
     const int ks = kseq % kStashRecs;
     if (kind == kStashKeep && kseq >= kStashRecs &&
-        !wait_phase(sh, &sh.kfree[ks], phase_of(kseq - kStashRecs)))
+        !warp_wait(sh, &sh.kfree[ks], phase_of(kseq - kStashRecs)))
       return;
     if (kind == kStashKeep) {
       ++kseq;
@@ -748,11 +759,10 @@ __device__ __forceinline__ void close_chunks(const StepParams& p,
   const int lane = threadIdx.x & 31;
   for (int seq = 0;; ++seq) {
     const int slot = seq % kStashRecs;
-    if (!wait_phase(sh, &sh.full[slot], phase_of(seq))) return;
+    if (!warp_wait(sh, &sh.full[slot], phase_of(seq))) return;
     const uint32_t kind = sh.rec[slot].kind;
     if (kind == kStashEnd) return;
-    if (!wait_phase(sh, &sh.done[slot], phase_of(seq))) return;
-    __syncwarp();
+    if (!warp_wait(sh, &sh.done[slot], phase_of(seq))) return;
     const Rec& r = sh.rec[slot];
     const int k = r.tensor, c = r.chunk, first = r.first, n = r.n_chunks;
     const bool again = n > (int)gridDim.x * q.max_keep;
