@@ -501,7 +501,14 @@ struct Worker {
     return true;
   }
 
+  // All the work; early if the launch gives up, with tiles still in the ring.
   __device__ __forceinline__ void run() {
+    take_all();
+    __syncwarp();
+    tmem_wait_st();   // no store may outlive the allocation
+  }
+
+  __device__ __forceinline__ void take_all() {
     for (int seq = 0;; ++seq) {
       const int rs = seq % kStashRecs;
       const Rec& r = sh.rec[rs];

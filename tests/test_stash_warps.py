@@ -1,7 +1,8 @@
 """The one-launch step's warps when a launch gives up: the device code of its
 workers, drawer and closer, cut from lamb_stash.cu and built for the host by
 tests/stash_warps.cpp with a thread for each lane.  Whatever moment a half of a
-warp learns of it at, the lanes of the warp leave together."""
+warp learns of it at, the lanes of the warp leave together, and none leaves a
+store to tensor memory in flight."""
 import os
 import shutil
 import subprocess
@@ -47,3 +48,7 @@ def _run(harness, scenario):
 @pytest.mark.parametrize("scenario", UNIFORM)
 def test_lanes_of_a_warp_leave_together(harness, scenario):
     _run(harness, scenario)
+
+
+def test_no_store_to_tensor_memory_outlives_its_worker(harness):
+    _run(harness, "worker_stores")
