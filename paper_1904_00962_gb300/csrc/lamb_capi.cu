@@ -148,7 +148,7 @@ struct lamb_plan {
   int64_t st_n_chunks = 0;      // its own chunk table
   ChunkDesc* st_chunks = nullptr;
   TensorDesc* st_tensors = nullptr;
-  float2* st_sums = nullptr;
+  double2* st_sums = nullptr;
   float2* st_gsums = nullptr;
   StashItem* st_items = nullptr;
   StashRec* st_recs = nullptr;
@@ -617,7 +617,7 @@ static lamb_status_t plan_create(const int64_t* sizes, int32_t n_tensors,
   const size_t o_oc_bar = carve(kBarWords * sizeof(uint32_t));
   const size_t o_st_chunks = carve(h_st_chunks.size() * sizeof(ChunkDesc));
   const size_t o_st_tensors = carve(h_st_tensors.size() * sizeof(TensorDesc));
-  const size_t o_st_slots = carve(h_st_chunks.size() * sizeof(float2));
+  const size_t o_st_sums = carve(h_st_chunks.size() * sizeof(double2));
   const size_t o_st_gsums = carve(h_st_chunks.size() * sizeof(float2));
   const size_t o_st_items = carve(h_items.size() * sizeof(StashItem));
   const size_t o_st_recs = carve(h_items.size() * sizeof(StashRec));
@@ -652,7 +652,7 @@ static lamb_status_t plan_create(const int64_t* sizes, int32_t n_tensors,
   p->oc_bar = reinterpret_cast<uint32_t*>(base + o_oc_bar);
   p->st_chunks = reinterpret_cast<ChunkDesc*>(base + o_st_chunks);
   p->st_tensors = reinterpret_cast<TensorDesc*>(base + o_st_tensors);
-  p->st_sums = reinterpret_cast<float2*>(base + o_st_slots);
+  p->st_sums = reinterpret_cast<double2*>(base + o_st_sums);
   p->st_gsums = reinterpret_cast<float2*>(base + o_st_gsums);
   p->st_items = reinterpret_cast<StashItem*>(base + o_st_items);
   p->st_recs = reinterpret_cast<StashRec*>(base + o_st_recs);
@@ -947,6 +947,7 @@ static int launch_two_pass_step(const lamb_plan* p, const StepParams& sp,
   if (stash_takes(p, sp.flags, lars)) {
     StashParams q;
     q.recs = p->st_recs;
+    q.sums = p->st_sums;
     q.words = p->st_words;
     q.bar = p->st_bar;
     q.n_items = p->st_n_items;
@@ -958,7 +959,6 @@ static int launch_two_pass_step(const lamb_plan* p, const StepParams& sp,
     StepParams own = sp;
     own.chunks = p->st_chunks;
     own.tensors = p->st_tensors;
-    own.slots = p->st_sums;
     own.n_chunks = (int32_t)p->st_n_chunks;
     own.grad_slots = p->st_gsums;
     int n = 0;

@@ -6,9 +6,9 @@
 // copy).  Here the SM that forms a chunk's u keeps it, with w, until the
 // tensor's ratio is known, and then writes the new w: 28 B.  The element
 // arithmetic is the two-pass kernels' (m, v and u are theirs bit for bit); the
-// norms are summed in another fixed order (fp32 over 20 elements of a thread,
-// fp32 trees over a chunk's warps, fp64 over chunks), so every run gives the
-// same bits.
+// norms are summed in another fixed order (fp32 over four elements of a thread,
+// two floats over the thread's tiles and the chunk's warps, fp64 over chunks), so
+// every run gives the same bits, and a norm is within some 2e-9 of the exact one.
 //
 // One cooperative launch, one CTA per SM, 20 warps:
 //   workers (16 warps)  A TILE is 1,024 elements of a chunk, one float4 for
@@ -75,6 +75,7 @@ constexpr int kWorkers = 2 * kWarps;
 constexpr int kDrawer = kWorkers, kCloser = kWorkers + 1,
               kPoller = kWorkers + 2, kLoader = kWorkers + 3;
 constexpr int kStashThreads = (kWorkers + 4) * 32;
+constexpr uint32_t kAllLanes = 0xffffffffu;
 constexpr int kStages = 3;       // pairs of tiles in flight
 constexpr int kTmemSlots = 32;   // float4s a thread has in tensor memory: 512
                                  // columns, 4 warps per quarter, 4 each
@@ -83,6 +84,42 @@ constexpr int kPairBytes = 2 * kStashTile * 4 + 16;
 template <typename GT>
 constexpr int kStageBytes = 3 * kPairBytes + 2 * kStashTile * (int)sizeof(GT) +
                             16;
+
+// ---------------------------------------------------------------------------
+// Sums of squares in two floats (the error of each addition is kept: ~48
+// significant bits), as in the on-chip kernel, whose plans run here too.  Not
+// renormalised on the way, so that hi alone is the fp32 sum, infinities
+// included.  Against plain fp32 sums, us: BERT-base 515 / 518, BERT-large 1512 /
+// 1496 (with more loads in flight in `combine`), 4,000 ragged tensors 4562 /
+// 4590.
+// ---------------------------------------------------------------------------
+struct Sum2 {
+  float hi, lo;
+};
+__device__ __forceinline__ void sum2_add(Sum2& a, float x) {
+  const float s = __fadd_rn(a.hi, x);
+  const float y = __fsub_rn(s, a.hi);
+  a.lo = __fadd_rn(a.lo, __fadd_rn(__fsub_rn(a.hi, __fsub_rn(s, y)),
+                                   __fsub_rn(x, y)));
+  a.hi = s;
+}
+__device__ __forceinline__ void sum2_add(Sum2& a, const Sum2& b) {
+  sum2_add(a, b.hi);
+  a.lo = __fadd_rn(a.lo, b.lo);
+}
+// Each half of the warp's lanes by itself: valid in lanes 0 and 16.
+__device__ __forceinline__ void sum2_half_warps(Sum2& a) {
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) {
+    const Sum2 b{__shfl_xor_sync(kAllLanes, a.hi, o),
+                 __shfl_xor_sync(kAllLanes, a.lo, o)};
+    sum2_add(a, b);
+  }
+}
+// (the error term of a sum that is not finite is not a number)
+__device__ __forceinline__ double sum2_value(const Sum2& a) {
+  return isfinite(a.hi) ? (double)a.hi + (double)a.lo : (double)a.hi;
+}
 
 // A kept chunk that waits for its update.
 struct __align__(16) Kept {
@@ -110,7 +147,7 @@ struct __align__(16) Rec : StashRec {
 struct Shared {
   Rec rec[kStashRecs];
   Kept kept[kStashRecs];
-  float2 red[kStashRecs][kWorkers];   // per worker: sum w^2, sum u^2
+  Sum2 red[kStashRecs][2][kWorkers];   // sum w^2, sum u^2 of each worker
   uint64_t full[kStashRecs];     // record written
   uint64_t done[kStashRecs];     // the workers finished pass 1 (or pass 2 of
                                  // a re-read chunk)
@@ -148,7 +185,6 @@ __device__ __forceinline__ bool wait_phase(const Shared& sh, uint64_t* b,
 // The same, and whether the launch gives up, with one answer for a warp: its
 // lanes look at the flag one by one, and lanes that left alone would be waited
 // for in the next warp-wide operation.
-constexpr uint32_t kAllLanes = 0xffffffffu;
 __device__ __forceinline__ bool warp_wait(const Shared& sh, uint64_t* b,
                                           uint32_t parity) {
   return __all_sync(kAllLanes, wait_phase(sh, b, parity));
@@ -283,7 +319,7 @@ struct Worker {
   int wslot = 0, held = 0;       // next ring slot, slots held
   int kseq = 0;                  // kept chunks formed
   int hseq = 0, htile, hslot = 0;   // oldest held one, its next tile
-  float aw = 0.f, au = 0.f;
+  Sum2 aw{0.f, 0.f}, au{0.f, 0.f};
 
   __device__ Worker(const StepParams& p, const StashParams& q, Shared& s,
                     char* m, uint32_t tmem)
@@ -383,6 +419,19 @@ struct Worker {
     return true;
   }
 
+  // The squares of a thread's elements of a tile.
+  __device__ __forceinline__ void add_squares(const float (&w)[4],
+                                              const float (&u)[4]) {
+    float qw = 0.f, qu = 0.f;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      qw = __fmaf_rn(w[c], w[c], qw);
+      qu = __fmaf_rn(u[c], u[c], qu);
+    }
+    sum2_add(aw, qw);
+    sum2_add(au, qu);
+  }
+
   // The full tile of the pair in stage `st`; false if the launch gives up.
   __device__ __forceinline__ bool full_tile(const Rec& r, int tile,
                                             const char* st, uint64_t* freed) {
@@ -427,11 +476,7 @@ struct Worker {
       if (kCopy) st_copy4(r.copy, at, o);
       return true;
     }
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      aw = __fmaf_rn(w[c], w[c], aw);
-      au = __fmaf_rn(u[c], u[c], au);
-    }
+    add_squares(w, u);
     return kind != kStashKeep || keep(w4, u4);
   }
 
@@ -474,12 +519,11 @@ struct Worker {
           }
         }
         u[c] = direction<kOpt>(m, v, g, w[c], r.lam, k);
-        aw = __fmaf_rn(w[c], w[c], aw);
-        au = __fmaf_rn(u[c], u[c], au);
       }
     }
     __syncwarp();
     if (lane == 0) mbar_arrive(freed);
+    add_squares(w, u);
     const float4 w4 = make_float4(w[0], w[1], w[2], w[3]);
     const float4 u4 = make_float4(u[0], u[1], u[2], u[3]);
     if (kind == kStashReread)
@@ -534,8 +578,15 @@ struct Worker {
         if ((tile & 2) && head_ready()) update_some();
       }
       if (kind != kStashReread) {
-        const float x = warp_sum(aw), y = warp_sum(au);
-        if (lane == 0) sh.red[rs][threadIdx.x >> 5] = make_float2(x, y);
+        // the lower lanes add w^2, the upper ones u^2
+        const bool up = lane >= 16;
+        Sum2 x = up ? au : aw;
+        const Sum2 y = up ? aw : au;
+        const Sum2 z{__shfl_xor_sync(kAllLanes, y.hi, 16),
+                     __shfl_xor_sync(kAllLanes, y.lo, 16)};
+        sum2_add(x, z);
+        sum2_half_warps(x);
+        if ((lane & 15) == 0) sh.red[rs][lane >> 4][threadIdx.x >> 5] = x;
       }
       if (kind == kStashKeep) ++kseq;
       __syncwarp();
@@ -543,7 +594,7 @@ struct Worker {
         mbar_arrive(&sh.done[rs]);
         mbar_arrive(&sh.free[rs]);
       }
-      aw = au = 0.f;
+      aw = au = Sum2{0.f, 0.f};
     }
     while (hseq < kseq) {
       if (!head_wait()) return;
@@ -726,40 +777,42 @@ __device__ __forceinline__ void draw(const StepParams& p, const StashParams& q,
 // ---------------------------------------------------------------------------
 // Closer
 // ---------------------------------------------------------------------------
-// Warp-wide sums of a tensor's slots in a fixed order, in fp64 as in the
-// two-pass finaliser; two rounds of eight slots per lane are in flight.
-__device__ __forceinline__ void combine(const float2* slots, int n, double* w,
-                                        double* u) {
-  constexpr int kLoads = 8;
+// Warp-wide sums of a tensor's slots (the x in lane 0, the y in lane 16) in a
+// fixed order, in fp64; two rounds of 16 loads per lane are in flight (BERT-base /
+// BERT-large, us: 8 loads 519.6 / 1500, 16 loads 518.0 / 1491).  A half warp for
+// each of the two sums: fp64 adds are slow, so no lane adds both, and none adds
+// the zeros past the last slot (a packed ragged list: 349 / 344 us).
+template <typename T2>
+__device__ __forceinline__ double combine(const T2* slots, int n) {
+  constexpr int kLoads = 16;
   const int lane = threadIdx.x & 31;
-  float2 x[kLoads], y[kLoads];
-  auto fetch = [&](float2 (&z)[kLoads], int base) {
+  const auto* from = &slots->x + (lane >> 4);
+  auto zero = slots->x;
+  zero = 0;
+  decltype(zero) x[kLoads], y[kLoads];
+  auto fetch = [&](decltype(zero) (&z)[kLoads], int base) {
 #pragma unroll
     for (int i = 0; i < kLoads; ++i) {
-      const int at = base + 32 * i + lane;
-      z[i] = at < n ? __ldcg(slots + at) : make_float2(0.f, 0.f);
+      const int at = base + 16 * i + (lane & 15);
+      z[i] = at < n ? __ldcg(from + 2 * at) : zero;
     }
   };
-  double a = 0.0, b = 0.0;
+  double a = 0.0;
   fetch(x, 0);
-  for (int base = 0; base < n; base += 32 * kLoads) {
-    fetch(y, base + 32 * kLoads);
+  for (int base = 0; base < n; base += 16 * kLoads) {
+    fetch(y, base + 16 * kLoads);
 #pragma unroll
     for (int i = 0; i < kLoads; ++i) {
-      a += (double)x[i].x;
-      b += (double)x[i].y;
+      if (base + 16 * i < n) a += (double)x[i];
       x[i] = y[i];
     }
   }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    a += __shfl_xor_sync(0xffffffffu, a, o);
-    b += __shfl_xor_sync(0xffffffffu, b, o);
-  }
-  *w = a;
-  *u = b;
+  for (int o = 8; o > 0; o >>= 1) a += __shfl_xor_sync(kAllLanes, a, o);
+  return a;
 }
 
+static_assert(kWorkers == 16, "half a warp adds the workers' sums");
 __device__ __forceinline__ void close_chunks(const StepParams& p,
                                              const StashParams& q, Shared& sh,
                                              double coef) {
@@ -773,30 +826,26 @@ __device__ __forceinline__ void close_chunks(const StepParams& p,
     const Rec& r = sh.rec[slot];
     const int k = r.tensor, c = r.chunk, first = r.first, n = r.n_chunks;
     const bool again = n > (int)gridDim.x * q.max_keep;
-    float2 x = make_float2(0.f, 0.f);
-    if (lane < kWorkers) x = sh.red[slot][lane];
+    Sum2 z = sh.red[slot][lane >> 4][lane & 15];
     __syncwarp();
     if (lane == 0) mbar_arrive(&sh.free[slot]);
     if (kind == kStashReread) continue;
-    x.x = warp_sum(x.x);
-    x.y = warp_sum(x.y);
-    double a, b;
-    if (n == 1) {   // the tensor's only chunk
-      a = (double)__shfl_sync(0xffffffffu, x.x, 0);
-      b = (double)__shfl_sync(0xffffffffu, x.y, 0);
-    } else {
+    sum2_half_warps(z);
+    double sum = sum2_value(z);   // of w^2 in lane 0, of u^2 in lane 16
+    if (n > 1) {
+      const double u2 = __shfl_sync(kAllLanes, sum, 16);
       int last = 0;
       if (lane == 0) {
         // releases the slot and, through the workers' barrier, their m and v
-        p.slots[c] = x;
+        q.sums[c] = make_double2(sum, u2);
         last = atom_add_acq_rel(&p.tickets[k], 1u) + 1u == (uint32_t)n;
         if (last) p.tickets[k] = 0u;
       }
       if (!__shfl_sync(0xffffffffu, last, 0)) continue;
-      combine(p.slots + first, n, &a, &b);
+      sum = combine(q.sums + first, n);
     }
-    const double root = sqrt(lane & 1 ? b : a);   // both at once
-    const double un = __shfl_sync(0xffffffffu, root, 1);
+    const double root = sqrt(sum);   // both at once
+    const double un = __shfl_sync(kAllLanes, root, 16);
     if (lane == 0) {
       const double wn = root;
       double rho = 1.0;                                // zero-norm rule
@@ -808,7 +857,7 @@ __device__ __forceinline__ void close_chunks(const StepParams& p,
       p.ratio[k] = rho;
       p.wnorm[k] = wn;
       p.unorm[k] = un;
-      if (!isfinite(a) || !isfinite(b)) atomicOr(p.status, kStatusNonfinite);
+      if (!isfinite(wn) || !isfinite(un)) atomicOr(p.status, kStatusNonfinite);
     }
   }
 }
@@ -1096,8 +1145,8 @@ __global__ void __launch_bounds__(kThreads)
       if (last) p.tickets[ch.tensor] = 0u;
     }
     if (!__shfl_sync(0xffffffffu, last, 0)) continue;
-    double sum, nan;
-    combine(p.grad_slots + td.first_chunk, td.n_chunks, &sum, &nan);
+    const double sum = combine(p.grad_slots + td.first_chunk, td.n_chunks);
+    const double nan = __shfl_sync(kAllLanes, sum, 16);
     int last_tensor = 0;
     if (lane == 0) {
       p.gsq[ch.tensor] = sum;

@@ -5,7 +5,7 @@
 // aligned):
 //   ChunkDesc  chunks[n_chunks]     16 B  its own chunk table
 //   TensorDesc tensors[n_tensors]   32 B  and tensor table
-//   float2     slots[n_chunks]       8 B  per chunk (sum w^2, sum u^2)
+//   double2    sums[n_chunks]       16 B  per chunk (sum w^2, sum u^2)
 //   float2     gsums[n_chunks]       8 B  per chunk (sum g^2, sum 0*g)
 //   StashItem  items[n_items]        8 B  the work, in the order it is drawn
 //   StashRec   recs[n_items]        64 B  the same with all that a CTA needs
@@ -73,6 +73,7 @@ constexpr int kStashBarWords = 128;
 
 struct StashParams {
   const StashRec* recs;
+  double2* sums;
   uint64_t* words;
   uint32_t* bar;
   int32_t n_items;

@@ -148,6 +148,8 @@ static void __threadfence() {}
 static float __uint_as_float(uint32_t x) { return of_bits<float>(x); }
 static uint32_t __float_as_uint(float x) { return (uint32_t)bits_of(x); }
 static float __double2float_rn(double x) { return (float)x; }
+static float __fadd_rn(float a, float b) { return a + b; }
+static float __fsub_rn(float a, float b) { return a - b; }
 static float __fmaf_rn(float a, float b, float c) { return std::fmaf(a, b, c); }
 
 namespace lamb {

@@ -238,6 +238,39 @@ def test_on_chip_plans_of_several_rounds(misalign):
     short.plan.destroy()
 
 
+@pytest.mark.parametrize("kind", ["on_chip", "two_pass"])
+@pytest.mark.parametrize("misalign", [None, {0, 4, 6}],
+                         ids=["aligned", "unaligned"])
+def test_norms_keep_more_than_fp32_sums(kind, misalign):
+    """||w|| and ||u|| against 64 bits, the u's elements being exact here (fp32,
+    no decay, no corrections).  Squares are added in fp32 over four elements
+    only: a norm of n elements is then within 2^-24 / sqrt(n) or so, 4.5e-10 on
+    average and 1.6e-9 at most over 400 tensors of 10,240 normal elements by a
+    host model; fp32 sums over a chunk gave 2.5e-8 and 6.7e-8.  An on-chip
+    plan's norms, in two floats, must not lose by AUTO's choice of kernel."""
+    sizes = [C] * 40 + [8192] * 20 + [3 * C + 5, 100001]
+    if kind == "two_pass":
+        sizes += [22 * C + 5]
+    r = Run(sizes, misalign=misalign, onchip_max_ctas=5)
+    assert r.plan.info()["algorithm"] == {
+        "on_chip": B.LAMB_ALGO_ON_CHIP,
+        "two_pass": B.LAMB_ALGO_TWO_PASS}[kind]
+    r.hyper = B.make_hyper(weight_decay=0., eps=2.0 ** -20,
+                           bias_correction=False)
+    r.step = r.plan.step_call("lamb", r.hyper, *r.scalars)
+    w = [r.st.download("w", k).astype(np.float64) for k in range(len(sizes))]
+    r.step()
+    _, wn, un = (x.cpu().numpy() for x in r.out()[1])
+    for k in range(len(sizes)):
+        u = r.st.download("m", k) / (np.sqrt(r.st.download("v", k)) +
+                                     np.float32(2.0 ** -20))
+        assert u.dtype == np.float32
+        for got, x in ((wn[k], w[k]), (un[k], u.astype(np.float64))):
+            want = np.sqrt(np.dot(x, x))
+            assert abs(got - want) <= 4e-9 * want, (k, got / want - 1)
+    r.plan.destroy()
+
+
 def test_a_layout_read_again_for_the_most_part_takes_the_two_launches():
     r = Run([60 * C, 5 * C], algorithm=B.LAMB_ALGO_AUTO, onchip_max_ctas=2)
     assert r.launches() == 2
