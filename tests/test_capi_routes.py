@@ -1,0 +1,69 @@
+"""What a step launches, for any layout and option: the C entry points' host
+code, built by tests/capi_routes.cpp on a stand-in for the CUDA runtime, with
+launchers that write down their calls."""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+from conftest import ROOT
+
+CSRC = os.path.join(ROOT, "paper_1904_00962_gb300", "csrc")
+AUTO, TWO_PASS, ON_CHIP = 0, 1, 3
+GRAD_NORM, SKIP = 0x8, 0x10
+TOO_LARGE = 720          # cudaErrorCooperativeLaunchTooLarge
+LAUNCH_FAILURE = 719     # cudaErrorLaunchFailure
+
+
+@pytest.fixture(scope="module")
+def routes(tmp_path_factory):
+    gxx = shutil.which("g++")
+    if gxx is None:
+        pytest.skip("g++ not available")
+    exe = tmp_path_factory.mktemp("capi_routes") / "capi_routes"
+    cmd = [gxx, "-std=c++17", "-O1", "-w",
+           "-I", os.path.join(ROOT, "include"), "-I", "/usr/local/cuda/include",
+           "-I", CSRC, "-x", "c++", os.path.join(CSRC, "lamb_capi.cu"),
+           os.path.join(CSRC, "planner.cpp"),
+           os.path.join(ROOT, "tests", "capi_routes.cpp"), "-o", str(exe)]
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    assert res.returncode == 0, res.stderr[-4000:]
+
+    def run(sizes, algorithm=AUTO, opt="lamb", flags=0, **options):
+        res = subprocess.run(
+            [str(exe), str(algorithm), opt, str(flags), sizes] +
+            [f"{k}={v}" for k, v in options.items()],
+            capture_output=True, text=True, timeout=60)
+        assert res.returncode == 0, res.stderr
+        return res.stdout.strip()
+    return run
+
+
+BIG = "1000000x200"      # AUTO: a two-pass plan that steps in one launch
+
+
+@pytest.mark.parametrize("opt", ["lamb", "nlamb", "nnlamb", "lars"])
+def test_a_refused_cooperative_launch_takes_the_two_kernels(routes, opt):
+    """Fewer SMs free to this process than the device has: the two launches need
+    no residency, the step succeeds and no error is left behind."""
+    line = routes(BIG, opt=opt, refuse=TOO_LARGE)
+    assert line == (f"algo 1 status 0: refused_{opt} {opt}1 {opt}2 timed 2 "
+                    "left 0")
+    line = routes(BIG, opt=opt)
+    assert line == f"algo 1 status 0: stash_{opt} timed 1 left 0"
+
+
+@pytest.mark.parametrize("flag", [GRAD_NORM, SKIP])
+def test_a_refused_launch_behind_the_gradient_check(routes, flag):
+    """The check has been launched by then; the two kernels form it again."""
+    line = routes(BIG, flags=flag, refuse=TOO_LARGE)
+    assert line == ("algo 1 status 0: check refused_lamb lamb1+gn lamb2+gn "
+                    "timed 2 left 0")
+    assert routes(BIG, flags=flag) == (
+        "algo 1 status 0: check stash_lamb timed 2 left 0")
+
+
+def test_another_launch_error_is_reported(routes):
+    line = routes(BIG, refuse=LAUNCH_FAILURE)
+    assert line.startswith("algo 1 status 3: refused_lamb timed 0")
