@@ -207,7 +207,10 @@ typedef struct {
 #define LAMB_ONCHIP_ROW_ELEMS 128
 #define LAMB_TAIL_CHUNK_ELEMS 2048
 
-/* Optional plan-creation knobs (pass NULL for defaults). */
+/* Optional plan-creation knobs (pass NULL for defaults).  A plan made by AUTO
+ * with chunk_elems, blocks_per_sm, tail_elems or onchip_rows set keeps the
+ * two-pass or on-chip kernels, which they shape, for every step: the one-launch
+ * form has its own chunks and grid. */
 typedef struct {
   int32_t chunk_elems;   /* two-pass: elements per chunk, multiple of 1024 in
                             [1024, 1<<24]; 0 = default (16384)             */

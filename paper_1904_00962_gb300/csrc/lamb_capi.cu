@@ -341,7 +341,10 @@ static lamb_status_t plan_create(const int64_t* sizes, int32_t n_tensors,
   int unmet_wait = 0, oc_max_ctas = 0, oc_rows_opt = 0;
   int64_t tail_opt = 0;
   int sh_world = 1, sh_rank = 0;
+  bool shaped = false;   // the caller shapes the two-pass or on-chip kernels
   if (opts) {
+    shaped = opts->chunk_elems || opts->blocks_per_sm || opts->tail_elems ||
+             opts->onchip_rows;
     if (opts->chunk_elems) chunk = opts->chunk_elems;
     if (opts->blocks_per_sm < 0)
       return fail(LAMB_ERR_INVALID_ARG, "blocks_per_sm < 0");
@@ -549,7 +552,9 @@ static lamb_status_t plan_create(const int64_t* sizes, int32_t n_tensors,
   std::vector<StashItem> h_items;
   std::vector<ChunkDesc> h_st_chunks;
   std::vector<TensorDesc> h_st_tensors;
-  if (auto_algo && sh_world == 1 &&
+  // A plan with options that the one launch has no use for keeps the kernels
+  // they are meant for.
+  if (auto_algo && sh_world == 1 && !shaped &&
       (algo == LAMB_ALGO_TWO_PASS || p->oc_n_rounds >= kStashMinRounds)) {
     rc = stash_prepare(device, p->grad_bf16, &p->st_slots, &p->st_wslots);
     if (rc) {

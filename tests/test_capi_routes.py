@@ -67,3 +67,25 @@ def test_a_refused_launch_behind_the_gradient_check(routes, flag):
 def test_another_launch_error_is_reported(routes):
     line = routes(BIG, refuse=LAUNCH_FAILURE)
     assert line.startswith("algo 1 status 3: refused_lamb timed 0")
+
+
+@pytest.mark.parametrize("option", [
+    {"chunk_elems": 4096}, {"blocks_per_sm": 1}, {"tail_elems": 65536}],
+    ids=lambda o: next(iter(o)))
+@pytest.mark.parametrize("opt", ["lamb", "lars", "nnlamb"])
+def test_options_of_the_two_kernels_keep_them(routes, opt, option):
+    """A caller who shapes the two-pass kernels gets them from AUTO, with the
+    chunks, the grid or the tail asked for."""
+    assert routes(BIG, opt=opt, **option) == (
+        f"algo 1 status 0: {opt}1 {opt}2 timed 2 left 0")
+
+
+def test_options_of_the_on_chip_kernel_keep_it(routes):
+    several = "100000x150"       # an on-chip plan of several rounds
+    assert routes(several) == "algo 3 status 0: stash_lamb timed 1 left 0"
+    for option in ({"onchip_rows": 200}, {"chunk_elems": 4096}):
+        assert routes(several, **option) == (
+            "algo 3 status 0: onchip_lamb timed 1 left 0")
+    # a limit on the CTAs is one of the one launch too
+    assert routes(several, onchip_max_ctas=100) == (
+        "algo 3 status 0: stash_lamb timed 1 left 0")
