@@ -792,24 +792,21 @@ __device__ __forceinline__ void draw(const StepParams& p, const StashParams& q,
 // ---------------------------------------------------------------------------
 // Closer
 // ---------------------------------------------------------------------------
-// Warp-wide sums of a tensor's slots (the x in lane 0, the y in lane 16) in a
-// fixed order, in fp64; two rounds of 16 loads per lane are in flight (BERT-base /
-// BERT-large, us: 8 loads 519.6 / 1500, 16 loads 518.0 / 1491).  A half warp for
-// each of the two sums: fp64 adds are slow, so no lane adds both, and none adds
-// the zeros past the last slot (a packed ragged list: 349 / 344 us).
-template <typename T2>
-__device__ __forceinline__ double combine(const T2* slots, int n) {
+// Warp-wide sums of a tensor's chunk sums (of w^2 in lane 0, of u^2 in lane 16)
+// in a fixed order, in fp64; two rounds of 16 loads per lane are in flight
+// (BERT-base / BERT-large, us: 8 loads 519.6 / 1500, 16 loads 518.0 / 1491).  A
+// half warp for each of the two: fp64 adds are slow, so no lane adds both, and
+// none adds the zeros past the last chunk (a packed ragged list: 349 / 344 us).
+__device__ __forceinline__ double combine(const double2* sums, int n) {
   constexpr int kLoads = 16;
   const int lane = threadIdx.x & 31;
-  const auto* from = &slots->x + (lane >> 4);
-  auto zero = slots->x;
-  zero = 0;
-  decltype(zero) x[kLoads], y[kLoads];
-  auto fetch = [&](decltype(zero) (&z)[kLoads], int base) {
+  const double* from = &sums->x + (lane >> 4);
+  double x[kLoads], y[kLoads];
+  auto fetch = [&](double (&z)[kLoads], int base) {
 #pragma unroll
     for (int i = 0; i < kLoads; ++i) {
       const int at = base + 16 * i + (lane & 15);
-      z[i] = at < n ? __ldcg(from + 2 * at) : zero;
+      z[i] = at < n ? __ldcg(from + 2 * at) : 0.0;
     }
   };
   double a = 0.0;
@@ -818,7 +815,7 @@ __device__ __forceinline__ double combine(const T2* slots, int n) {
     fetch(y, base + 16 * kLoads);
 #pragma unroll
     for (int i = 0; i < kLoads; ++i) {
-      if (base + 16 * i < n) a += (double)x[i];
+      if (base + 16 * i < n) a += x[i];
       x[i] = y[i];
     }
   }
@@ -1123,6 +1120,42 @@ __device__ __forceinline__ int check_vec(const __nv_bfloat16* g, int len,
   return len & ~3;
 }
 
+// Warp-wide sums of a tensor's slots in a fixed order, in fp64 as in the
+// two-pass finaliser; two rounds of eight slots per lane are in flight.  (With
+// `combine` above in its place the kernel gets fewer registers, and with fp32 g
+// it waits for its loads one by one: 31 / 48 us on 6M parameters.)
+__device__ __forceinline__ void combine_slots(const float2* slots, int n,
+                                              double* sum, double* nan) {
+  constexpr int kLoads = 8;
+  const int lane = threadIdx.x & 31;
+  float2 x[kLoads], y[kLoads];
+  auto fetch = [&](float2 (&z)[kLoads], int base) {
+#pragma unroll
+    for (int i = 0; i < kLoads; ++i) {
+      const int at = base + 32 * i + lane;
+      z[i] = at < n ? __ldcg(slots + at) : make_float2(0.f, 0.f);
+    }
+  };
+  double a = 0.0, b = 0.0;
+  fetch(x, 0);
+  for (int base = 0; base < n; base += 32 * kLoads) {
+    fetch(y, base + 32 * kLoads);
+#pragma unroll
+    for (int i = 0; i < kLoads; ++i) {
+      a += (double)x[i].x;
+      b += (double)x[i].y;
+      x[i] = y[i];
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    a += __shfl_xor_sync(kAllLanes, a, o);
+    b += __shfl_xor_sync(kAllLanes, b, o);
+  }
+  *sum = a;
+  *nan = b;
+}
+
 template <typename GT>
 __global__ void __launch_bounds__(kThreads)
     grad_check_kernel(const StepParams p, int needs_t) {
@@ -1160,8 +1193,8 @@ __global__ void __launch_bounds__(kThreads)
       if (last) p.tickets[ch.tensor] = 0u;
     }
     if (!__shfl_sync(0xffffffffu, last, 0)) continue;
-    const double sum = combine(p.grad_slots + td.first_chunk, td.n_chunks);
-    const double nan = __shfl_sync(kAllLanes, sum, 16);
+    double sum, nan;
+    combine_slots(p.grad_slots + td.first_chunk, td.n_chunks, &sum, &nan);
     int last_tensor = 0;
     if (lane == 0) {
       p.gsq[ch.tensor] = sum;
