@@ -144,7 +144,9 @@ struct lamb_plan {
   int st_n_items = 0;
   int64_t st_wait_ns = 0;
   int st_extra = 0;
-  double st_again = 0.0;        // share of the chunks that is read again
+  // which steps it pays for (one_launch_pays): LAMB, N-LAMB and NN-LAMB, LARS,
+  // LAMB to NN-LAMB with the gradient check, with the skip mode
+  bool st_pays[5] = {false, false, false, false, false};
   int64_t st_n_chunks = 0;      // its own chunk table
   ChunkDesc* st_chunks = nullptr;
   TensorDesc* st_tensors = nullptr;
@@ -321,6 +323,66 @@ lamb_status_t lamb_layout_rounds(const int64_t* sizes, int32_t n_tensors,
     ++i;
   }
   return LAMB_OK;
+}
+
+// Where one launch pays against two, from what either was measured to take on a
+// GB300 (us, two launches / one).  An element saves 12 B (LARS 8, N-LAMB also its
+// g), which is the gain of those that are kept without further ado, `easy` here,
+// and a step saves about 8 us of the second launch and of ramps.  Against that:
+//   hard    a tensor larger than the `most` chunks that the SMs keep stalls them
+//           while its ratio is formed, and what is read again (`again` elements)
+//           costs more than in a pass of its own: LARS 10 x 6.5M 267 / 355, 1 x
+//           8M 49 / 54, BERT-base 436 / 444, but BERT-large 1302 / 1220; LAMB
+//           10 x 6.5M 387 / 402, 10 x 10M 587 / 635, 1 x 14M 97 / 105, but 1 x 8M
+//           77 / 61 and BERT-base 635 / 518; N-LAMB 10 x 9M 575 / 548, 40 x 8M
+//           1945 / 1967.  (One chunk more than fits is harmless: 161 tensors of
+//           65.3M parameters, three of them 609 chunks, LARS 266 / 256)
+//   nearly  a tensor nearly that large leaves the SMs little else to do: LARS
+//           10 x 5.6M 230 / 244, 10 x 5M 212 / 198
+//   short   chunks cost an SM about 1 us each: LARS 100,000 x 500 1229 / 1338, x
+//           3,000 1776 / 1799, x 3,500 1921 / 1839 (LAMB, x 500: 1768 / 1370)
+//   check   the launch that reads g takes 18 us (bf16 12) and 0.6 (0.3) us per 1M
+//           elements, where the two launches form its sums on the way and only
+//           the skip mode reads g again.  LAMB, check / skip mode: f32, one
+//           tensor of 6M 61 / 73 and 65 / 73, a BERT of two layers and 9.6M 83 /
+//           97 and 87 / 97, 161 tensors of 10.5M 88 / 88 and 99 / 88, ResNet-50
+//           171 / 152 and 195 / 152; bf16, 6M 60 / 61 and 64 / 61, 10.5M 87 / 78
+//           and 98 / 78.  The two launches' check is paid for by the chunk, short
+//           or not: 20,000 x 500 and 10M 801 / 477
+// The lines below are those gains and costs in elements; `kept` is what the SMs
+// keep, 6.2M elements on 152 of them.
+static void one_launch_pays(const int64_t* sizes, int32_t n, int64_t most,
+                            int grad_bf16, bool* pays) {
+  const double kept = (double)(most * kStashChunk);
+  double total = 0, again = 0, easy = 0, chunks = 0;
+  double hard = 0, nearly = 0, nearly_n = 0;
+  for (int32_t k = 0; k < n; ++k) {
+    const int64_t c = (sizes[k] + kStashChunk - 1) / kStashChunk;
+    const double d = (double)sizes[k];
+    total += d;
+    if (c > most) again += d - kept;
+    if (c > most + most / 64) {
+      hard += 1;
+    } else if (8 * c > 7 * most) {
+      nearly_n += 1;
+      nearly += d;
+    } else {
+      easy += d;
+      chunks += (double)c;
+    }
+  }
+  const bool most_once = again <= 0.4 * total;
+  pays[0] = most_once &&
+            easy + nearly + 0.83 * kept >= 0.1 * hard * kept + 0.77 * again;
+  pays[1] = most_once;
+  pays[2] = easy >= 3500.0 * chunks &&
+            easy + 3.0 * kept >=
+                (3.2 * hard + 0.8 * nearly_n) * kept + 5.0 * again;
+  const double checked = chunks * kStashChunk + nearly + 0.83 * kept -
+                         (0.1 * hard + 0.47 * nearly_n +
+                          (grad_bf16 ? 1.55 : 2.3)) * kept - 0.77 * again;
+  pays[3] = most_once && checked >= (grad_bf16 ? 0.14 : 0.3) * total;
+  pays[4] = most_once && checked >= 0.0;
 }
 
 static lamb_status_t plan_create(const int64_t* sizes, int32_t n_tensors,
@@ -583,8 +645,8 @@ static lamb_status_t plan_create(const int64_t* sizes, int32_t n_tensors,
       p->st_max_keep = keep;
       p->st_n_chunks = count;
       p->st_n_items = (int)h_items.size();
-      // chunks that go through pass 1 alone and are taken again for the update
-      p->st_again = (double)(h_items.size() - (size_t)count) / (double)count;
+      one_launch_pays(sizes, n_tensors, (int64_t)ctas * keep, p->grad_bf16,
+                      p->st_pays);
       p->st_wait_ns = wait_ms * 1000000;
       p->st_extra = unmet_wait;
     } else {
@@ -927,19 +989,18 @@ static int launch_onchip_step(const lamb_plan* p, const StepParams& sp,
 }
 
 // Does the one-launch form run this step (after a launch that reads g alone,
-// with the gradient check or the skip mode)?  Not where too much of the layout
-// has to be read again after all: that part runs at about 0.8 of the
-// two launches' rate (one launch / two, us: 200 tensors of 1M, none again, LAMB
-// 877 / 1207, LARS 694 / 827; one of 10M, 0.4 again, 73 / 85 and 62 / 63; 40 of
-// 8M, 0.45 again, 1950 / 1914 and 1648 / 1313; one of 30M, 0.8 again, 209 / 205
-// and 176 / 143).  LARS has 8 B/parameter to win and the check's read of g
-// takes 2 or 4 of them: with it the two launches stay (76.8M parameters in 161
-// tensors, bf16 g: 335 in one launch behind the check, 304 in two).
-static bool stash_takes(const lamb_plan* p, uint32_t flags, bool lars) {
-  return p->st_grid > 0 &&
-         !(lars && p->algorithm == LAMB_ALGO_ON_CHIP) &&
-         !(lars && (flags & (LAMB_FLAG_GRAD_NORM | LAMB_FLAG_SKIP_NONFINITE))) &&
-         p->st_again <= (lars ? 0.2 : 0.4);
+// with the gradient check or the skip mode)?  opt as below.  LARS keeps the two
+// launches on a plan that AUTO made on-chip, as before there was one (ResNet-50
+// 109 us, one launch 101; 161 tensors of 10.5M parameters 57 and 53), and with
+// the check, whose read of g takes what it would win (76.8M parameters in 161
+// tensors, bf16 g: 304 us in two, 335 behind the check).
+static bool stash_takes(const lamb_plan* p, uint32_t flags, int opt) {
+  if (p->st_grid == 0) return false;
+  const bool skip = (flags & LAMB_FLAG_SKIP_NONFINITE) != 0;
+  const bool check = skip || (flags & LAMB_FLAG_GRAD_NORM) != 0;
+  if (opt == 3)
+    return !check && p->algorithm != LAMB_ALGO_ON_CHIP && p->st_pays[2];
+  return p->st_pays[check ? (skip ? 4 : 3) : (opt ? 1 : 0)];
 }
 
 // The two launches of a two-pass step, or one (stash_takes).  opt: 0 LAMB, 1
@@ -949,7 +1010,7 @@ static int launch_two_pass_step(const lamb_plan* p, const StepParams& sp,
                                 cudaEvent_t* ev) {
   const bool lars = opt == 3;
   int rc = 0;
-  if (stash_takes(p, sp.flags, lars)) {
+  if (stash_takes(p, sp.flags, opt)) {
     StashParams q;
     q.recs = p->st_recs;
     q.sums = p->st_sums;
@@ -1006,7 +1067,7 @@ static lamb_status_t launch_step(lamb_plan* p, const StepParams& sp, int opt,
     const cudaError_t e = cudaEventRecord(ev[0], stream);
     if (e != cudaSuccess) return cuda_fail(e, what);
   }
-  const int n = !stash_takes(p, sp.flags, opt == 3) &&
+  const int n = !stash_takes(p, sp.flags, opt) &&
                         onchip_takes(p, sp.flags, opt == 3)
                     ? launch_onchip_step(p, sp, opt, stream, ev)
                     : launch_two_pass_step(p, sp, opt, stream, ev);

@@ -89,3 +89,44 @@ def test_options_of_the_on_chip_kernel_keep_it(routes):
     # a limit on the CTAs is one of the one launch too
     assert routes(several, onchip_max_ctas=100) == (
         "algo 3 status 0: stash_lamb timed 1 left 0")
+
+
+# What a step launches where one launch was measured to pay and where not (a
+# GB300, us; see one_launch_pays).
+@pytest.mark.parametrize("opt,sizes,one", [
+    ("lars", "1000000x200", True),                  # 827 / 694
+    ("lars", "1000000x300,30000000", True),         # 1287 / 1192
+    ("lars", "1000000x50,9400000", True),           # 244 / 228
+    ("lars", "4000x20000,6000000", True),           # 447 / 413
+    ("lars", "6500000x10", False),                  # 267 / 355
+    ("lars", "8000000", False),                     # 49 / 54
+    ("lars", "1000000x100,30000000", False),        # 517 / 537
+    ("lars", "5600000x10", False),                  # 230 / 244
+    ("lars", "500x100000", False),                  # 1229 / 1338
+    ("lars", "2000x2000,6000000", False),           # 63 / 66
+    ("lamb", "500x100000", True),                   # 1768 / 1370
+    ("lamb", "8000000", True),                      # 77 / 61
+    ("lamb", "1000000x100,30000000", True),         # 753 / 626
+    ("lamb", "10000000x10", False),                 # 587 / 635
+    ("lamb", "6500000x10", False),                  # 387 / 402
+    ("lamb", "14000000", False),                    # 97 / 105
+    ("nlamb", "9000000x10", True),                  # 575 / 548
+    ("nlamb", "30000000", False),                   # 212 / 229
+])
+def test_one_launch_where_it_pays(routes, opt, sizes, one):
+    want = f"stash_{opt} timed 1" if one else f"{opt}1 {opt}2 timed 2"
+    assert routes(sizes, opt=opt) == f"algo 1 status 0: {want} left 0"
+
+
+@pytest.mark.parametrize("flag,sizes,one", [
+    (GRAD_NORM, "1000000x20,10000000,1000000x20", True),
+    (GRAD_NORM, "500x20000,10000000", True),        # 801 / 477
+    (GRAD_NORM, "6000000", False),                  # 61 / 73
+    (GRAD_NORM, "10000000", False),                 # 86 / 109
+    (SKIP, "6000000", False),                       # 65 / 73
+    (SKIP, "1000000x20,10000000", True),            # 225 / 192
+])
+def test_one_launch_behind_the_check_where_it_pays(routes, flag, sizes, one):
+    want = "check stash_lamb" if one else "lamb1+gn lamb2+gn"
+    assert routes(sizes, flags=flag) == (
+        f"algo 1 status 0: {want} timed 2 left 0")
