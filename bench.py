@@ -60,6 +60,8 @@ BYTES_PASS2 = 4 + 4 + 4 + 4 + 2          # read m,v,w ; write w, copy = 18
 BYTES_STEP = BYTES_PASS1 + BYTES_PASS2   # 40
 BYTES_SINGLE_TOUCH = 2 + 12 + 12 + 2     # 28
 ALGO_CODES = {"auto": 0, "two_pass": 1, "on_chip": 3}
+OPT_CODES = {"lamb": 0, "lars": 1, "nlamb": 2, "nnlamb": 3}   # LAMB_OPT_*
+FORM_NAMES = {1: "two_pass", 3: "on_chip", 4: "one_launch"}   # LAMB_FORM_*
 # the committed ncu summaries holding measured DRAM traffic per launch, per
 # (algorithm, layout, optimizer), and the kernel sources they were taken on
 TWO_PASS_SOURCES = ("lamb_kernels.cu", "lamb_device.cuh", "lamb_internal.h")
@@ -141,14 +143,6 @@ def one_launch_model(opt, gb, cb, variant="plain"):
     if variant in ("grad_norm", "skip_nonfinite"):
         return [f"grad_check_kernel<g{8 * gb}>"] + names, [gb] + per
     return names, per
-
-
-def one_launch_on_chip_plan(sizes, n_rounds):
-    """AUTO's rule for an on-chip plan of several rounds: three rounds or
-    more and chunks (10,240 elements at most) of 5,400 elements on average
-    step in one launch over all tensors instead of round by round."""
-    chunks = sum(-(-s // 10240) for s in sizes)
-    return n_rounds >= 3 and sum(sizes) >= 5400 * chunks
 
 
 def noalloc_overhead(st, L, hyper, d_step, d_lr, stream, one_step, n=20):
@@ -623,19 +617,23 @@ def run_ours(args):
     plan = LambPlan(st, L.decay, algorithm=ALGO_CODES[args.algo],
                     chunk_elems=args.chunk_elems)
     info = plan.info()
-    algo = info["algorithm"]
-    if args.algo == "auto" and opt == "lars" and algo == 3 and \
-            info["n_rounds"] > 1:
-        algo = 1   # AUTO runs LARS over several rounds on the two-pass kernels
-    streamed = 0
-    if algo == 3:
-        cap = info["grid_blocks"] * info["rows_per_cta"] * info["row_elems"]
-        streamed = sum(s for s in L.sizes if s > cap)
-    kernel_names, kernel_bytes = kernel_model(
-        opt, algo, 2 if L.grad_dtype == "bf16" else 4,
-        2 if L.copy_dtype == "bf16" else 0, args.variant, streamed / P)
-    profile = PROFILES.get((algo, args.layout, opt)) if (
-        args.variant == "plain" and args.layers == 24) else None
+    form = B.lamb_plan_step_form(plan.handle, hyper, OPT_CODES[opt])
+    gb = 2 if L.grad_dtype == "bf16" else 4
+    cb = 2 if L.copy_dtype == "bf16" else 0
+    if form == B.LAMB_FORM_ONE_LAUNCH:
+        kernel_names, kernel_bytes = one_launch_model(opt, gb, cb,
+                                                      args.variant)
+        profile = (STASH_PROFILE, f"{args.layout}/{opt}", STASH_SOURCES)
+    else:
+        streamed = 0
+        if form == B.LAMB_FORM_ON_CHIP:
+            cap = info["grid_blocks"] * info["rows_per_cta"] * info["row_elems"]
+            streamed = sum(s for s in L.sizes if s > cap)
+        kernel_names, kernel_bytes = kernel_model(opt, form, gb, cb,
+                                                  args.variant, streamed / P)
+        profile = PROFILES.get((form, args.layout, opt))
+    if args.variant != "plain" or args.layers != 24:
+        profile = None
     d_step = torch.ones(1, dtype=torch.int64, device=dev)
     d_lr = torch.full((1,), float(np.float32(h.lr)), dtype=torch.float32,
                       device=dev)
@@ -696,24 +694,6 @@ def run_ours(args):
     ms_instr = e0.elapsed_time(e1)
     n_timed, ms_kernels = B.lamb_plan_read_timing(plan.handle, 3)
     B.lamb_plan_set_timing(plan.handle, False)
-    # AUTO's one-launch form: a plain step of a two-pass plan is then one
-    # kernel; an on-chip plan's step is one kernel either way
-    B.lamb_plan_set_timing(plan.handle, True)
-    plan.step_call(opt, layout_hyper(L, opt, "plain")[1], d_step, d_lr,
-                   d_prod if opt in ("nlamb", "nnlamb") else None, 0.004,
-                   stream)()
-    barrier()
-    n_plain = sum(ms > 0 for ms in B.lamb_plan_read_timing(plan.handle, 3)[1])
-    B.lamb_plan_set_timing(plan.handle, False)
-    lars_check = lars and args.variant in ("grad_norm", "skip_nonfinite")
-    if args.algo == "auto" and n_plain == 1 and not lars_check and (
-            algo == 1 or (opt != "lars" and one_launch_on_chip_plan(
-                L.sizes, info["n_rounds"]))):
-        kernel_names, kernel_bytes = one_launch_model(
-            opt, 2 if L.grad_dtype == "bf16" else 4,
-            2 if L.copy_dtype == "bf16" else 0, args.variant)
-        profile = (STASH_PROFILE, f"{args.layout}/{opt}", STASH_SOURCES) if (
-            args.variant == "plain" and args.layers == 24) else None
     # The first K timed steps are the measurement.  When the two regions take
     # less than CLOCK_WINDOW_S, the same K-step region runs again (each timed
     # the same way) until the clock sampler has watched the GPU for that long,
@@ -839,10 +819,8 @@ def run_ours(args):
         if profile else None
     ms_step = ms_total / args.steps
     step_bytes = sum(kernel_bytes)
-    single_bytes = single_touch_bytes(opt, 2 if L.grad_dtype == "bf16" else 4,
-                                      2 if L.copy_dtype == "bf16" else 0)
-    two_bytes = two_pass_bytes(opt, 2 if L.grad_dtype == "bf16" else 4,
-                               2 if L.copy_dtype == "bf16" else 0)
+    single_bytes = single_touch_bytes(opt, gb, cb)
+    two_bytes = two_pass_bytes(opt, gb, cb)
     step_gbs = step_bytes * P / (ms_step * 1e-3) / 1e9
 
     cpu = None
@@ -902,7 +880,7 @@ def run_ours(args):
         "single_touch_bytes_per_param": single_bytes,
         "frac_of_peak_single_touch_model": single_bytes * P /
         (ms_step * 1e-3) / 1e9 / peak,
-        "algorithm": {1: "two_pass", 3: "on_chip"}[algo],
+        "algorithm": FORM_NAMES[form],
         "kernels": {kernel_names[i]: {"ms_per_launch": per_launch_ms[i],
                                       "alg_bytes_per_param": kernel_bytes[i]}
                     for i in range(len(kernel_names))},
@@ -974,8 +952,7 @@ def run_shard(args):
     L = get_layout(args.layout)
     opt = args.optimizer
     h, hyper = layout_hyper(L, opt)
-    code = {"lamb": B.LAMB_OPT_LAMB, "lars": B.LAMB_OPT_LARS,
-            "nlamb": B.LAMB_OPT_NLAMB, "nnlamb": B.LAMB_OPT_NNLAMB}[opt]
+    code = OPT_CODES[opt]
     psi = 0.004
     st = DeviceState(L.sizes, grad_dtype=L.grad_dtype,
                      copy_dtype=L.copy_dtype, device=dev,

@@ -413,7 +413,26 @@ LAMB_API lamb_status_t lamb_plan_copy_trust_ratios(lamb_plan_t plan, double* rat
 LAMB_API lamb_status_t lamb_plan_query(lamb_plan_t plan, uint32_t* status_bits,
                               int32_t clear, cudaStream_t stream);
 
+/* What the plan was made with.  `algorithm` is what AUTO chose, or the option;
+ * the chunk, grid and round fields describe that algorithm's kernels.  A step
+ * may run in another form: lamb_plan_step_form. */
 LAMB_API lamb_status_t lamb_plan_get_info(lamb_plan_t plan, lamb_plan_info_t* info);
+
+/* Host-only: which kernels a step of this plan runs.
+ *   hyper      of the step (of its flags the gradient check and the skip mode
+ *              matter); NULL: a step without flags
+ *   optimizer  LAMB_OPT_*
+ *   form       receives LAMB_FORM_*
+ * (Where a one-launch step is refused because this process has fewer SMs than
+ * the device, the two-pass kernels run in its place.)  Errors: INVALID_ARG. */
+#define LAMB_FORM_TWO_PASS 1    /* the two streaming kernels                */
+#define LAMB_FORM_ON_CHIP 3     /* the on-chip kernel (streamed tensors
+                                   through the two-pass kernels first)      */
+#define LAMB_FORM_ONE_LAUNCH 4  /* AUTO's one launch (with the gradient check
+                                   or the skip mode behind one that reads g) */
+LAMB_API lamb_status_t lamb_plan_step_form(lamb_plan_t plan,
+                                           const lamb_hyper_t* hyper,
+                                           int32_t optimizer, int32_t* form);
 
 /* Instrumentation: when enabled, each step records CUDA events on its
  * stream around every kernel it launches (up to 4096 steps are kept).

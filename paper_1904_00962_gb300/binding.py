@@ -48,7 +48,7 @@ LAMB_STATUS_SKIPPED = 0x10
 
 EXPORTED = ["lamb_plan_create", "lamb_plan_bind", "lamb_step", "lars_step",
             "lamb_plan_trust_ratios", "lamb_plan_copy_trust_ratios",
-            "lamb_plan_query", "lamb_plan_get_info",
+            "lamb_plan_query", "lamb_plan_get_info", "lamb_plan_step_form",
             "lamb_plan_set_timing", "lamb_plan_read_timing",
             "lamb_plan_destroy", "lamb_layout_chunks", "lamb_last_error",
             "lamb_abi_version", "lamb_step_noalloc",
@@ -86,6 +86,9 @@ LAMB_OPT_LAMB = 0
 LAMB_OPT_LARS = 1
 LAMB_OPT_NLAMB = 2
 LAMB_OPT_NNLAMB = 3
+LAMB_FORM_TWO_PASS = 1
+LAMB_FORM_ON_CHIP = 3
+LAMB_FORM_ONE_LAUNCH = 4
 LAMB_STATUS_WAIT_TIMEOUT = 0x4
 
 
@@ -145,6 +148,8 @@ def load(path: str | None = None) -> ctypes.CDLL:
     lib.lamb_plan_copy_grad_norms.argtypes = [vp, vp, vp, vp, vp]
     lib.lamb_plan_query.argtypes = [vp, POINTER(c_uint32), c_int32, vp]
     lib.lamb_plan_get_info.argtypes = [vp, POINTER(lamb_plan_info_t)]
+    lib.lamb_plan_step_form.argtypes = [vp, POINTER(lamb_hyper_t), c_int32,
+                                        POINTER(c_int32)]
     lib.lamb_plan_set_timing.argtypes = [vp, c_int32]
     lib.lamb_plan_read_timing.argtypes = [vp, POINTER(c_int32),
                                           POINTER(c_double), c_int32]
@@ -346,6 +351,14 @@ def lamb_plan_get_info(plan) -> dict:
     info = lamb_plan_info_t()
     _check(load().lamb_plan_get_info(c_void_p(plan), byref(info)))
     return {name: getattr(info, name) for name, _ in info._fields_}
+
+
+def lamb_plan_step_form(plan, hyper: lamb_hyper_t, optimizer) -> int:
+    """Which kernels a step runs: LAMB_FORM_*."""
+    form = c_int32()
+    _check(load().lamb_plan_step_form(c_void_p(plan), byref(hyper),
+                                      int(optimizer), byref(form)))
+    return form.value
 
 
 def lamb_plan_set_timing(plan, enable=True) -> None:

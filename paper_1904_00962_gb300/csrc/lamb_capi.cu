@@ -1383,6 +1383,20 @@ lamb_status_t lamb_plan_get_info(lamb_plan_t plan, lamb_plan_info_t* info) {
   return LAMB_OK;
 }
 
+lamb_status_t lamb_plan_step_form(lamb_plan_t plan, const lamb_hyper_t* hyper,
+                                  int32_t optimizer, int32_t* form) {
+  if (!plan || !form) return fail(LAMB_ERR_INVALID_ARG, "NULL argument");
+  if (optimizer < LAMB_OPT_LAMB || optimizer > LAMB_OPT_NNLAMB)
+    return fail(LAMB_ERR_INVALID_ARG, "unknown optimizer %d", optimizer);
+  const int opt = optimizer == LAMB_OPT_LARS ? 3
+                  : optimizer >= LAMB_OPT_NLAMB ? optimizer - 1 : 0;
+  const uint32_t flags = hyper ? hyper->flags : 0u;
+  *form = stash_takes(plan, flags, opt) ? LAMB_FORM_ONE_LAUNCH
+          : onchip_takes(plan, flags, opt == 3) ? LAMB_FORM_ON_CHIP
+                                                : LAMB_FORM_TWO_PASS;
+  return LAMB_OK;
+}
+
 lamb_status_t lamb_plan_set_timing(lamb_plan_t plan, int32_t enable) {
   if (!plan) return fail(LAMB_ERR_INVALID_ARG, "plan is NULL");
   const size_t n_events = (size_t)kMaxTimedSteps * (kKernelsPerStep + 1);

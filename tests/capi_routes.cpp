@@ -38,6 +38,11 @@ int two_pass(const std::string& name, const lamb::StepParams& p) {
   return seen(name + ((p.flags & (LAMB_FLAG_GRAD_NORM |
                                   LAMB_FLAG_SKIP_NONFINITE)) ? "+gn" : ""));
 }
+bool seen_any(const char* prefix) {
+  for (const std::string& x : g_launches)
+    if (x.rfind(prefix, 0) == 0) return true;
+  return false;
+}
 const char* kNames[4] = {"lamb", "nlamb", "nnlamb", "lars"};
 }  // namespace
 
@@ -180,6 +185,14 @@ int main(int argc, char** argv) {
   h.eps = 1e-6;
   h.trust_coef = 1.;
   h.flags = flags;
+  const int32_t optimizer = opt == "lamb" ? LAMB_OPT_LAMB
+                            : opt == "lars" ? LAMB_OPT_LARS
+                            : opt == "nlamb" ? LAMB_OPT_NLAMB : LAMB_OPT_NNLAMB;
+  int32_t form = 0;
+  if (lamb_plan_step_form(plan, &h, optimizer, &form) ||
+      !lamb_plan_step_form(plan, &h, 4, &form) ||
+      !lamb_plan_step_form(plan, &h, optimizer, nullptr))
+    return die("form");
   int64_t step = 1;
   float lr = .1f;
   double prod = 1.;
@@ -193,6 +206,11 @@ int main(int argc, char** argv) {
   int32_t timed = 0;
   double ms[3] = {0., 0., 0.};
   if (lamb_plan_read_timing(plan, &timed, ms, 3)) return die("read timing");
+  // what the step launched is what the plan said it would
+  const bool one = seen_any("stash_") || seen_any("refused_");
+  if (form != (one ? LAMB_FORM_ONE_LAUNCH
+               : seen_any("onchip_") ? LAMB_FORM_ON_CHIP : LAMB_FORM_TWO_PASS))
+    return die("form of the step");
   std::string line = "algo " + std::to_string(info.algorithm) + " status " +
                      std::to_string((int)st) + ":";
   for (const std::string& x : g_launches) line += " " + x;

@@ -387,6 +387,7 @@ def test_null_plan_is_rejected(lib):
                lambda: B.lamb_plan_bind(0, [1], [1], [1]),
                lambda: B.lamb_plan_query(0),
                lambda: B.lamb_plan_get_info(0),
+               lambda: B.lamb_plan_step_form(0, h, B.LAMB_OPT_LAMB),
                lambda: B.lamb_plan_copy_trust_ratios(0)):
         with pytest.raises(B.LambError) as ei:
             fn()
