@@ -145,17 +145,20 @@ def one_launch_model(opt, gb, cb, variant="plain"):
     return names, per
 
 
-def noalloc_overhead(st, L, hyper, d_step, d_lr, stream, one_step, n=20):
+def noalloc_overhead(st, L, hyper, d_step, d_lr, stream, n=20):
     """Device time and host enqueue time per call of lamb_step_noalloc
-    against the plan's lamb_step, on the same state, n calls each after
-    three of each untimed.  The no-alloc call rebuilds its tables on the
-    device every call; the difference is its per-call overhead."""
+    against lamb_step of a two-pass plan, whose kernels it runs, on the same
+    state, n calls each after three of each untimed.  The no-alloc call
+    rebuilds its tables on the device every call; the difference is its
+    per-call overhead."""
     from ctypes import byref, c_int64, c_uint8, c_void_p
 
     import torch
     from paper_1904_00962_gb300 import binding as B
-    from paper_1904_00962_gb300.state import _dtype_code
+    from paper_1904_00962_gb300.state import LambPlan, _dtype_code
     lib = B.load()
+    plan = LambPlan(st, L.decay, algorithm=B.LAMB_ALGO_TWO_PASS)
+    step = plan.step_call("lamb", hyper, d_step, d_lr, stream=stream)
     k = L.n_tensors
     sizes = (c_int64 * k)(*[int(x) for x in L.sizes])
     mask = (c_uint8 * k)(*[1 if d else 0 for d in L.decay])
@@ -173,9 +176,9 @@ def noalloc_overhead(st, L, hyper, d_step, d_lr, stream, one_step, n=20):
 
     for _ in range(3):
         na()
-        one_step()
+        step()
     res = {}
-    for name, fn in (("plan", one_step), ("noalloc", na)):
+    for name, fn in (("plan", step), ("noalloc", na)):
         e0 = torch.cuda.Event(enable_timing=True)
         e1 = torch.cuda.Event(enable_timing=True)
         torch.cuda.synchronize()
@@ -187,6 +190,7 @@ def noalloc_overhead(st, L, hyper, d_step, d_lr, stream, one_step, n=20):
         e1.record(stream)
         e1.synchronize()
         res[name] = (e0.elapsed_time(e1) / n, (t1 - t0) / n * 1e6)
+    plan.destroy()
     return {"calls": n, "ms_per_call": res["noalloc"][0],
             "plan_ms_per_call": res["plan"][0],
             "overhead_ms": res["noalloc"][0] - res["plan"][0],
@@ -797,8 +801,7 @@ def run_ours(args):
     noalloc = None
     if rank == 0 and opt == "lamb" and args.variant == "plain":
         try:
-            noalloc = noalloc_overhead(st, L, hyper, d_step, d_lr, stream,
-                                       one_step)
+            noalloc = noalloc_overhead(st, L, hyper, d_step, d_lr, stream)
         except B.LambError as e:   # beyond the entry point's limits
             noalloc = {"unavailable": str(e)}
 
