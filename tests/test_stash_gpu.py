@@ -67,6 +67,9 @@ class Run:
                         torch.full((1,), f32(2e-3), device=dev),
                         torch.full((1,), .6, dtype=torch.float64, device=dev))
         self.step = self.plan.step_call(opt, self.hyper, *self.scalars)
+        self.form = B.lamb_plan_step_form(
+            self.plan.handle, self.hyper,
+            ["lamb", "lars", "nlamb", "nnlamb"].index(opt))
 
     def launches(self):
         B.lamb_plan_set_timing(self.plan.handle, True)
@@ -108,6 +111,7 @@ def test_one_launch_matches_the_two_pass_kernels(opt, grad, copy, misalign,
     one = Run(SIZES, algorithm=B.LAMB_ALGO_AUTO, **kw)
     two = Run(SIZES, algorithm=B.LAMB_ALGO_TWO_PASS, **kw)
     w0 = two.st.w.clone()
+    assert one.form == B.LAMB_FORM_ONE_LAUNCH
     assert one.launches() == 1 and two.launches() == 2
     assert one.plan.info()["algorithm"] == B.LAMB_ALGO_TWO_PASS
     (w1, *s1), r1 = one.out()
@@ -139,7 +143,7 @@ def _grad_norms(r):
     return gn.cpu().numpy(), float(total.item()), int(bad.item())
 
 
-@pytest.mark.parametrize("opt", ["lamb", "lars", "nnlamb"])
+@pytest.mark.parametrize("opt", ["lamb", "nnlamb"])
 @pytest.mark.parametrize("grad,copy", [("f32", None), ("bf16", "bf16")])
 @pytest.mark.parametrize("misalign", [None, {0, 5, 8, 13, 18, 21}],
                          ids=["aligned", "unaligned"])
@@ -148,16 +152,18 @@ def _grad_norms(r):
 def test_gradient_check_matches_the_two_pass_kernels(opt, grad, copy, misalign,
                                                      bad, flag):
     """The check reads g in its own launch; norms, decision, status word and
-    what a skipped step leaves and reports are those of the two kernels."""
+    what a skipped step leaves and reports are those of the two kernels.  (Both
+    are two launches: the sums tell them apart.)"""
     runs = []
-    for algo in (B.LAMB_ALGO_AUTO, B.LAMB_ALGO_TWO_PASS):
+    for algo, form in ((B.LAMB_ALGO_AUTO, B.LAMB_FORM_ONE_LAUNCH),
+                       (B.LAMB_ALGO_TWO_PASS, B.LAMB_FORM_TWO_PASS)):
         r = Run(SIZES, opt=opt, grad=grad, copy=copy, misalign=misalign,
                 flags={flag: True, "lr_schedule": (2e-3, 10, 100)},
                 algorithm=algo, onchip_max_ctas=5)
         if bad is not None:
             r.st.view("g", 20)[100002] = bad
         before = r.out()[0]
-        assert r.launches() == 2
+        assert r.form == form and r.launches() == 2
         after, res = r.out()
         runs.append((before, after, res, _grad_norms(r), r.plan.query()))
         r.plan.destroy()
@@ -174,6 +180,8 @@ def test_gradient_check_matches_the_two_pass_kernels(opt, grad, copy, misalign,
     np.testing.assert_allclose(n1[1], n2[1], rtol=2 * TOL_RATIO)
     for a, b in zip(r1, r2):
         np.testing.assert_allclose(a.cpu(), b.cpu(), rtol=2 * TOL_RATIO)
+    # ||w||: two floats over a chunk against fp32 sums
+    assert not torch.equal(r1[1], r2[1])
 
 
 @pytest.mark.parametrize("flag", ["grad_norm", "skip_nonfinite"])
@@ -214,7 +222,7 @@ def test_on_chip_plans_of_several_rounds(misalign):
     two = Run(sizes, algorithm=B.LAMB_ALGO_TWO_PASS, **kw)
     info = one.plan.info()
     assert info["algorithm"] == B.LAMB_ALGO_ON_CHIP and info["n_rounds"] > 1
-    assert one.launches() == 1 and two.launches() == 2
+    assert one.form == B.LAMB_FORM_ONE_LAUNCH and one.launches() == 1 and two.launches() == 2
     (w1, *s1), r1 = one.out()
     (w2, *s2), r2 = two.out()
     assert _same(s1, s2)
@@ -229,10 +237,11 @@ def test_on_chip_plans_of_several_rounds(misalign):
     for r in (one, two):
         r.plan.destroy()
     lars = Run(sizes, opt="lars", algorithm=B.LAMB_ALGO_AUTO, **kw)
-    assert lars.launches() == 2
+    assert lars.form == B.LAMB_FORM_TWO_PASS and lars.launches() == 2
     lars.plan.destroy()
     short = Run([900] * 400, algorithm=B.LAMB_ALGO_AUTO, onchip_max_ctas=4)
-    assert short.plan.info()["n_rounds"] > 1 and short.launches() == 1
+    assert short.plan.info()["n_rounds"] > 1
+    assert short.form == B.LAMB_FORM_ON_CHIP and short.launches() == 1
     rho, wn, un = short.out()[1]
     assert not torch.equal(rho * un, wn)     # fp32: the on-chip kernel
     short.plan.destroy()
