@@ -25,8 +25,11 @@
  * g is float32 or bfloat16; an optional bfloat16 copy of the new w is written
  * with round-to-nearest-even.  All tensor pointers are DEVICE pointers on the
  * plan's device.  Pointers aligned to 16 bytes (8 bytes for bfloat16 arrays)
- * take the vectorised path; others are handled element by element (AUTO's
- * one-launch steps stream them in whole 16-byte granules all the same).
+ * take the vectorised path; others are handled element by element.  (AUTO's
+ * one-launch steps read whole 16-byte granules: of an array that does not start
+ * or end on one also the up to 15 bytes of memory in front of its first element
+ * or behind its last that share a granule with it.  They are not used, and no
+ * other granule is touched.)
  *
  * Ownership: the caller owns w, g, m, v, the bf16 copy, the step counter,
  * the learning rate and the streams.  The plan owns its chunk table, pointer
@@ -170,20 +173,22 @@ typedef struct {
                                      lars_step over more than one round runs
                                      the two-pass kernels
                                      (lamb_plan_get_info reports the choice).
-                                     A two-pass plan made by AUTO runs its
-                                     steps as ONE launch (behind one that
-                                     reads g, with the gradient check or the
-                                     skip mode; lars_step with either keeps
-                                     the two kernels) where most of the layout fits
-                                     the SMs in turn: a chunk's w and u stay
-                                     on the SM until its tensor's ratio is
-                                     known (28 B of HBM traffic per
-                                     parameter).  m,
-                                     v and u are the two kernels' bit for bit;
-                                     the norms are summed in another fixed
-                                     order.  So does an on-chip plan made
+                                     A two-pass plan made by AUTO runs a step
+                                     as ONE launch (behind one that reads g,
+                                     with the gradient check or the skip
+                                     mode; lars_step with either keeps the
+                                     two kernels) where that is the faster
+                                     way, for the most part where the layout
+                                     fits the SMs in turn: a chunk's w and u
+                                     stay on the SM until its tensor's ratio
+                                     is known (28 B of HBM traffic per
+                                     parameter).  m, v and u are the two
+                                     kernels' bit for bit; the norms are
+                                     summed in another fixed order and to
+                                     more bits.  So does an on-chip plan made
                                      by AUTO with several rounds and mostly
-                                     long tensors (lamb_step, nlamb_step)   */
+                                     long tensors (lamb_step, nlamb_step).
+                                     lamb_plan_step_form tells               */
 #define LAMB_ALGO_TWO_PASS 1      /* two streaming kernels per step: 40 B of
                                      HBM traffic per parameter (bf16 g/copy) */
 /* 2 is not assigned (plan creation rejects it)                           */
@@ -326,9 +331,13 @@ LAMB_API lamb_status_t lamb_plan_bind(lamb_plan_t plan, void* const* w,
  * steps of two plans at the same time on different streams (a wait that
  * cannot be met gives up after wait_limit_ms with LAMB_STATUS_WAIT_TIMEOUT
  * and leaves the plan unusable).  AUTO's one-launch steps are cooperative
- * launches too; steps of two such plans on different streams take turns, as
- * the device starts a cooperative grid only as a whole.  Steps of one plan,
- * like all steps, must not overlap. */
+ * launches too, of one CTA with nearly all of the shared memory on every SM: such
+ * a step starts when kernels of other streams leave that room on every SM, and
+ * steps of two such plans on different streams take turns, as the device starts
+ * a cooperative grid only as a whole.  Their CTAs wait for each other as well: a wait that gives up (wait_limit_ms,
+ * LAMB_STATUS_WAIT_TIMEOUT; never expected) leaves some tensors with their new w
+ * and others with only m and v updated, and the plan unusable.  LAMB_ALGO_TWO_PASS
+ * has neither condition.  Steps of one plan, like all steps, must not overlap. */
 LAMB_API lamb_status_t lamb_step(lamb_plan_t plan, const lamb_hyper_t* hyper,
                         int64_t* d_step, const float* d_lr,
                         cudaStream_t stream);
@@ -345,7 +354,7 @@ LAMB_API lamb_status_t lars_step(lamb_plan_t plan, const lamb_hyper_t* hyper,
 /* One N-LAMB step (appendix Algorithm 3: Nesterov momentum in the first
  * moment) or, with nesterov_second_moment = 1, one NN-LAMB step (Algorithm
  * 4: also in the second moment), over every tensor.  Uses w, g, m, v and
- * the two-pass kernels, or the on-chip kernel on an on-chip plan.
+ * the kernels that lamb_step takes (lamb_plan_step_form).
  *   hyper          beta1, beta2, eps, weight_decay, phi as for lamb_step;
  *                  the bias-correction flag is ignored (the Nesterov forms
  *                  carry their own corrections); INCREMENT_STEP honoured
@@ -561,9 +570,11 @@ LAMB_API lamb_status_t lamb_layout_rounds(
  *                      chunks; closes the step (INCREMENT_STEP, schedule,
  *                      N-LAMB product) like lamb_step.
  * The results on each rank's range, and the trust ratios, are bitwise equal
- * to one unsharded step of the same layout and tail.  The gradients of the
- * rank's range must be reduced (e.g. reduce-scattered) before pass 1, and
- * the new w gathered after pass 2, by the caller.  The kernels touch only
+ * to one unsharded step of a LAMB_ALGO_TWO_PASS plan of the same layout,
+ * chunk_elems and tail (AUTO's other forms sum the norms in another order: m
+ * and v are the same bits, w and the ratios agree to rounding).  The gradients
+ * of the rank's range must be reduced (e.g. reduce-scattered) before pass 1,
+ * and the new w gathered after pass 2, by the caller.  The kernels touch only
  * the rank's elements of w, g, m, v and the copy.  Not taken: GRAD_NORM,
  * SKIP_NONFINITE (INVALID_ARG).  Both halves are capturable; no timing
  * events are recorded for them.

@@ -84,10 +84,10 @@ __device__ __forceinline__ void cta_sum(float* x, float (*red)[kWarps]) {
 // warp 0 the warps, in fixed trees.  Spreading the slots over the whole CTA
 // keeps a tensor of thousands of chunks (BERT's word embedding: 1,908) to
 // one batch of L2 loads per thread.  Resets the ticket.  What bounds it: load
-// latency, then fp64 issue (all 398 tensors of BERT-large in one launch:
-// 12.3 us with one load in flight and every warp in the trees, 8.8 us so).  With the gradient
-// check (kGn) it also forms the tensor's sum g^2 and whether any of its
-// elements was Inf/NaN, and counts the tensor done.
+// latency, then fp64 issue (all 391 tensors of BERT-large in one launch:
+// 12.3 us with one load in flight and every warp in the trees, 8.8 us so).
+// With the gradient check (kGn) it also forms the tensor's sum g^2 and whether
+// any of its elements was Inf/NaN, and counts the tensor done.
 template <bool kGn>
 __device__ __noinline__ void finalize_tensor(const StepParams& p, int k,
                                              int first, int n, double coef) {
@@ -652,7 +652,7 @@ __global__ void __launch_bounds__(kThreads)
 // Every tensor's norms and trust ratio from the complete chunk slots (a
 // sharded step, after the slots were exchanged): one CTA per tensor, the
 // same fixed-order combine as the finaliser of pass 1, so the results equal
-// an unsharded step's bit for bit.
+// an unsharded two-pass step's bit for bit.
 __global__ void __launch_bounds__(kThreads)
     finalize_all_kernel(const StepParams p, double coef) {
   // one CTA per tensor, as when pass 1 finalises it: the same sums

@@ -14,13 +14,14 @@
 //   workers (16 warps)  A TILE is 1,024 elements of a chunk, one float4 for
 //     each of 256 threads; workers 0-7 take a chunk's even tiles and 8-15 its
 //     odd ones (8 warps alone were bound by the latency of the square root and
-//     the division: 2.5 ms on BERT-large).  A pair of tiles arrives in a stage of shared memory; after pass 1 w and u go to the
-//     thread's place in a ring of tiles, u in tensor memory, w in shared
-//     memory or, past its end, in tensor memory too (a warp reaches its own
-//     quarter of the lanes, which is all it needs: a thread's elements are
-//     read by nobody else).  Workers never meet: a warp has its own positions
-//     in the chunk sequence and in the ring, and updates w from the ring once
-//     a chunk's ratio is there, between the tiles of a later chunk.
+//     the division: 2.5 ms on BERT-large).  A pair of tiles arrives in a stage
+//     of shared memory; after pass 1 w and u go to the thread's place in a ring
+//     of tiles, u in tensor memory, w in shared memory or, past its end, in
+//     tensor memory too (a warp reaches its own quarter of the lanes, which is
+//     all it needs: a thread's elements are read by nobody else).  Workers never
+//     meet: a warp has its own positions in the chunk sequence and in the ring,
+//     and updates w from the ring once a chunk's ratio is there, between the
+//     tiles of a later chunk.
 //   loader   copies the pairs of tiles, one cp.async.bulk per array (issuing a
 //     copy takes ~100 cycles of the one warp), as far ahead as there are
 //     stages.  It copies whole 16-byte granules, so a tensor at any address
@@ -36,8 +37,8 @@
 //     record) and hands eta rho_k to the workers.
 //
 // Storage: w and u of a tile take 4 KB each.  Shared memory holds three stages
-// and 28 tiles of w next to the records (30 with bf16 g), tensor memory 64
-// tiles: a ring of 46 tiles, half of them even ones.  A CTA can always keep
+// and 28 tiles of w next to the records (32 with bf16 g), tensor memory 64
+// tiles: a ring of 46 tiles (48), half of them even ones.  A CTA can always keep
 // four chunks of 10,240 elements of one tensor: 6.2M parameters over 152 SMs.
 // A larger tensor (a word embedding) keeps its first chunks; the rest goes
 // through pass 1 only and is read again, last chunk first, when its ratio is
@@ -54,8 +55,8 @@
 // abort word, and every CTA returns.
 //
 // Measured (us per step, the two kernels / this one): BERT-large LAMB with bf16
-// g and copy 1924 / 1510, N-LAMB 2039 / 1515, BERT-base LAMB 638 / 518, 4,000
-// ragged tensors (1.1e9 parameters) 6416 / 4561.  That is 0.92 of a copy's rate
+// g and copy 1924 / 1496, N-LAMB 2039 / 1499, BERT-base LAMB 638 / 518, 4,000
+// ragged tensors (1.1e9 parameters) 6416 / 4590.  That is 0.93 of a copy's rate
 // on BERT-large's 28 B per parameter.  What is left there: the embedding's
 // second read, rings that are full while a 4096 x 1024 tensor is finished (13%
 // of the workers' time), and the last chunks' ratios.

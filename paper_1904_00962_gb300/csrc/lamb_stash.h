@@ -26,11 +26,13 @@ namespace lamb {
 constexpr int kStashTile = 4 * kThreads;   // elements: one float4 per thread
 // Elements per chunk.  A chunk is kept until its tensor's last one is done, so
 // short chunks need less room (of a 4096 x 1024 tensor an SM holds 27 tiles, and
-// what it forms while the last chunk is summed); but each takes a draw and a
-// ticket.  us per step, BERT-base / BERT-large / 4,000 ragged tensors: 8,192
-// elements 510 / 1612 / 4659, 10,240 508 / 1544 / 4581, 12,288 508 / 1628 / 4667,
-// 16,384 516 / 1743 / 4869; an odd number of tiles 5-15% slower (workers take
-// them in pairs).
+// what it forms while the last chunk is summed), and more of a tensor larger than
+// the SMs is kept; but each takes a draw, a tree of sums and a ticket.  us per
+// step, a two-layer encoder / BERT-base / BERT-large / 4,000 ragged tensors: 8,192
+// elements 67.9 / 538 / 1524 / 4695, 10,240 67.4 / 518 / 1493 / 4590, 12,288 69.1 /
+// 511 / 1479 / 4566, 16,384 64.6 / 506 / 1524 / 4600.  12,288 would keep 5.6M
+// parameters of a tensor in place of 6.2M, and the lines of AUTO's rules were
+// measured at 10,240.  Workers take tiles in pairs: the number is even.
 constexpr int kStashChunk = 10 * kStashTile;
 constexpr int kStashRecs = 16;   // chunks a CTA has drawn and not finished
 
